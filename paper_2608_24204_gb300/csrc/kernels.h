@@ -26,6 +26,9 @@ struct Bufs {
     float *fd_part;   // flash-decode split states                           [nkv][splits][group][d + 4]
     uint32_t *mega_bound; // persistent decode: row-share boundaries (2^24 = all) [num_sms + 1]
     float *mega_time;     // persistent decode: gate/up time per CTA, last step (us) [num_sms]
+    // persistent decode: words that carry a tag beside their value, all of them zero at first
+    uint64_t *tags;   // the region they share
+    uint64_t *tqkv, *tpart, *to, *txo, *txd, *tm;  // [nqkv], split states, [qdim], [H], [H], [F]
     float2 *rope;     // (cos, sin) of p * theta^(-2i/d)                     [max_tokens][d/2]
     int *pages;       // logical -> physical KV page                         [max_pages]
     int *tok;         // prefill chunk tokens                                [max_chunk]
@@ -38,9 +41,8 @@ struct Bufs {
     // 8-bit block format only: the matrix of the next prefill GEMM dequantised
     // as three bf16 terms (exact: a code times an fp16 scale has <= 18 significant bits)
     uint16_t *Wt[kTerms]; //                                                    [wt_elems]
-    // qk_norm only: k of this decode step before its norm and RoPE            [kvdim]
-    // and the prefill chunk's q | k before their norms and RoPE               [max_chunk][qdim + kvdim]
-    float *kraw, *QKraw;
+    // qk_norm only: the prefill chunk's q | k before their norms and RoPE     [max_chunk][qdim + kvdim]
+    float *QKraw;
 };
 
 // TMA descriptors of the prefill GEMM operands (built once per context).
@@ -73,6 +75,9 @@ struct LaunchHook {
 int fd_splits(int max_pages);
 size_t fd_part_floats(int nkv, int group, int d, int max_pages);
 
+// Words of the persistent step's attention split states.
+size_t mega_part_words(int nkv, int group, int d);
+
 // One-time per-process kernel attributes (dynamic shared memory limits).
 cudaError_t setup_kernels();
 
@@ -87,8 +92,9 @@ cudaError_t enqueue_lm_head_argmax_raw(const uint16_t *W, const uint16_t *gain, 
 bool decode_is_persistent(const Plan &p);
 
 // Whole decode step for the token in ctrl[CTRL_TOKEN] at position ctrl[CTRL_POS]:
-// 5 launches per layer + the LM head.  `pdl` enables programmatic dependent launch.
-cudaError_t enqueue_decode_step(const Plan &p, const Bufs &b, cudaStream_t st, bool pdl,
+// one persistent launch, or 5 launches per layer + the LM head (`pdl` enables programmatic
+// dependent launch between them).  map_kv: the KV pool's tensor map.
+cudaError_t enqueue_decode_step(const Plan &p, const Bufs &b, const CUtensorMap &map_kv, cudaStream_t st, bool pdl,
                                 LaunchHook *hook);
 
 // Final RMSNorm + LM head + argmax of the row in b.x; the last CTA writes

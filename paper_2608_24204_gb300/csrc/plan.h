@@ -47,9 +47,10 @@ struct Plan {
     // workspace (byte offsets)
     size_t ws_ctrl, ws_hist, ws_x, ws_q, ws_o, ws_m, ws_logits, ws_amax, ws_rope,
         ws_pages, ws_tok, ws_X, ws_fd_part, ws_mega_bound, ws_mega_time;
+    size_t ws_tags, tag_bytes;   // the persistent decode step's tagged words
     size_t ws_Q[3], ws_A[3], ws_O[3], ws_M[3];   // one buffer per bf16 term
     size_t ws_Wt[3];        // 8-bit format only: one matrix dequantised as three bf16 terms (prefill)
-    size_t ws_kraw, ws_QKraw;   // qk_norm only: this step's k before its norm (decode), the chunk's q|k (prefill)
+    size_t ws_QKraw;        // qk_norm only: the chunk's q|k before their norms (prefill)
     size_t wt_elems;        // elements of the largest per-layer matrix
     size_t ws_bytes;
     int num_sms;

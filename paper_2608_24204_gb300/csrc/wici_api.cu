@@ -144,6 +144,10 @@ const char *wici::make_plan(const wici_config *cfg, int num_sms, Plan *p) {
     P.ws_fd_part = ws(fd_part_floats(P.nkv, P.group, P.d, P.max_pages) * sizeof(float));
     P.ws_mega_bound = ws(((size_t)P.num_sms + 1) * sizeof(uint32_t));
     P.ws_mega_time = ws((size_t)P.num_sms * sizeof(float));
+    // tagged words (32-byte aligned arrays): q|k|v, residual after O and after down, o, m, split states
+    P.tag_bytes = ((size_t)P.nqkv + 2 * align_up(H, 4) + align_up(P.qdim, 4) + align_up(F, 4) +
+                   mega_part_words(P.nkv, P.group, P.d)) * sizeof(uint64_t);
+    P.ws_tags = ws(P.tag_bytes);
     P.ws_rope = ws((size_t)c.max_tokens * (P.d / 2) * sizeof(float2));
     P.ws_pages = ws((size_t)P.max_pages * 4);
     P.ws_tok = ws(T * 4);
@@ -157,7 +161,6 @@ const char *wici::make_plan(const wici_config *cfg, int num_sms, Plan *p) {
     P.wt_elems = 0;
     for (size_t e : {(size_t)P.nqkv * H, H * (size_t)P.qdim, 2 * F * H, H * F}) P.wt_elems = e > P.wt_elems ? e : P.wt_elems;
     for (int t = 0; t < kTerms; ++t) P.ws_Wt[t] = P.q8 ? ws(P.wt_elems * 2) : 0;
-    P.ws_kraw = P.qk_norm ? ws((size_t)P.kvdim * 4) : 0;
     P.ws_QKraw = P.qk_norm ? ws(T * (size_t)(P.qdim + P.kvdim) * 4) : 0;
     P.ws_bytes = w;
     return nullptr;
@@ -179,6 +182,13 @@ static Bufs make_bufs(const Plan &p, void *W, void *KV, void *WS) {
     b.fd_part = (float *)(ws + p.ws_fd_part);
     b.mega_bound = (uint32_t *)(ws + p.ws_mega_bound);
     b.mega_time = (float *)(ws + p.ws_mega_time);
+    b.tags = (uint64_t *)(ws + p.ws_tags);
+    b.tqkv = b.tags;
+    b.txo = b.tqkv + p.nqkv;   // nqkv is a multiple of head_dim
+    b.txd = b.txo + align_up(p.H, 4);
+    b.to = b.txd + align_up(p.H, 4);
+    b.tm = b.to + align_up(p.qdim, 4);
+    b.tpart = b.tm + align_up(p.F, 4);
     b.rope = (float2 *)(ws + p.ws_rope);
     b.pages = (int *)(ws + p.ws_pages);
     b.tok = (int *)(ws + p.ws_tok);
@@ -190,7 +200,6 @@ static Bufs make_bufs(const Plan &p, void *W, void *KV, void *WS) {
         b.M[t] = (uint16_t *)(ws + p.ws_M[t]);
         b.Wt[t] = p.q8 ? (uint16_t *)(ws + p.ws_Wt[t]) : nullptr;
     }
-    b.kraw = p.qk_norm ? (float *)(ws + p.ws_kraw) : nullptr;
     b.QKraw = p.qk_norm ? (float *)(ws + p.ws_QKraw) : nullptr;
     return b;
 }
@@ -335,6 +344,8 @@ int wici_create(const wici_config *cfg, void *cuda_stream, void *weight_dev, voi
              (e = cudaEventCreateWithFlags(&c->step_done[1], cudaEventDisableTiming)) != cudaSuccess))
             break;
         if ((e = cudaMemsetAsync(c->bufs.ctrl, 0, CTRL_WORDS * sizeof(int), c->stream)) != cudaSuccess) break;
+        // no word carries a step's tag (never zero in the first 2^32 / L steps)
+        if ((e = cudaMemsetAsync(c->bufs.tags, 0, p.tag_bytes, c->stream)) != cudaSuccess) break;
         // cache slots past the length are read (and weighted by zero) by the
         // tensor-core attention: they must hold finite values from the start
         if ((e = cudaMemsetAsync(c->bufs.KV, 0, p.kv_elems * 2, c->stream)) != cudaSuccess) break;
@@ -537,7 +548,8 @@ static int finish_call(wici_ctx *c, int32_t new_kv_len, int32_t *token_out) {
         cudaMemcpyAsync(c->bufs.ctrl + CTRL_ERR, c->pinned + 3, sizeof(int), cudaMemcpyHostToDevice, c->stream);
         cudaMemcpyAsync(c->bufs.ctrl + CTRL_POS, c->pinned + 4, sizeof(int), cudaMemcpyHostToDevice, c->stream);
         cudaMemsetAsync(c->bufs.ctrl + CTRL_LM_TICKET, 0, sizeof(int), c->stream);
-        cudaMemsetAsync(c->bufs.ctrl + CTRL_GRID_BAR, 0, sizeof(int), c->stream);
+        // the step that gave up is run again under the same tags: none of its words may stay
+        cudaMemsetAsync(c->bufs.tags, 0, c->plan.tag_bytes, c->stream);
         cudaMemsetAsync(c->bufs.ctrl + CTRL_ATTN_TICKET0, 0, 64 * sizeof(int), c->stream);
         cudaStreamSynchronize(c->stream);
         return fail(c, WICI_E_TIMEOUT, "a device-side wait gave up (site %d)", errw);
@@ -578,7 +590,7 @@ static int ensure_graph(wici_ctx *c) {
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        cudaError_t e2 = enqueue_decode_step(c->plan, c->bufs, cap, true, nullptr);
+        cudaError_t e2 = enqueue_decode_step(c->plan, c->bufs, c->maps.kv, cap, true, nullptr);
         e = cudaStreamEndCapture(cap, &g);
         if (e2 != cudaSuccess) e = e2;
     }
@@ -622,7 +634,7 @@ static cudaError_t launch_step(wici_ctx *c) {
     if (c->plan.cfg.max_sms > 0 && decode_is_persistent(c->plan)) {
         cudaEvent_t ev = c->step_done[c->steps_launched % kShareDepth];
         cudaError_t e = c->steps_launched >= kShareDepth ? cudaEventSynchronize(ev) : cudaSuccess;
-        if (e == cudaSuccess) e = enqueue_decode_step(c->plan, c->bufs, c->stream, false, nullptr);
+        if (e == cudaSuccess) e = enqueue_decode_step(c->plan, c->bufs, c->maps.kv, c->stream, false, nullptr);
         if (e == cudaSuccess) e = cudaEventRecord(ev, c->stream);
         if (e == cudaSuccess) ++c->steps_launched;
         return e;
@@ -743,7 +755,7 @@ int wici_profile_decode(wici_ctx *c, int32_t n_steps, const char **names, int32_
     EventHook hook;
     hook.st = c->stream;
     for (int i = 0; i < n_steps; ++i) {
-        cudaError_t e = enqueue_decode_step(c->plan, c->bufs, c->stream, false, &hook);
+        cudaError_t e = enqueue_decode_step(c->plan, c->bufs, c->maps.kv, c->stream, false, &hook);
         if (e != cudaSuccess) return fail(c, WICI_E_CUDA, "profile launch: %s", cudaGetErrorString(e));
     }
     int rc = finish_call(c, c->kv_len + n_steps, nullptr);
