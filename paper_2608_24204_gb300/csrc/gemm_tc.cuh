@@ -33,6 +33,13 @@
 //               columns each (one output row per thread), group sums in
 //               registers, then the fused epilogue on column pairs.  The
 //               epilogue of one tile overlaps the MMAs of the next.
+//
+// Few tiles (short chunks): the tiles of a 128-row chunk of a 4096-column matrix
+// are 32, on 152 SMs, and streaming the weights is what costs.  With SPLIT = 2 or 4
+// a cluster of SPLIT CTAs shares one tile: each takes a range of the k-blocks, then
+// the CTAs exchange column slices of their sums through shared memory (every CTA
+// adds the slices of its BN / SPLIT columns in rank order) and run the epilogue on
+// their slices.
 // Every mbarrier wait is bounded; a wait that gives up records its site in
 // *err and the CTA still drains its copies, frees TMEM and exits.
 #pragma once
@@ -62,6 +69,28 @@ struct TcTile {
     static constexpr uint32_t ACC_STRIDE = TC_TMEM_COLS / 2;              // TMEM columns between the two buffers
     static_assert(STAGES >= 3, "at least three ring stages");
 };
+
+// Tensor maps of one GEMM, all with boxes 64 elements wide and 128-byte swizzle.  One
+// copy per operand and k-block: boxes of 64 rows of W, three to a 192-column tile,
+// cost 17% of a long chunk's gate/up GEMM.
+struct GemmMaps {
+    CUtensorMap a[kTerms];   // activation terms, boxes of a_rows rows
+    CUtensorMap w[kTerms];   // weight terms, boxes of BN rows
+    int a_rows;              // 128, or what a chunk shorter than a tile needs
+};
+
+// everything the cluster's CTAs wrote before is visible to all of them after
+__device__ __forceinline__ void cluster_sync_all() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+// 16 bytes into the shared memory of CTA `rank` of the cluster, at the address that `addr` has here
+__device__ __forceinline__ void st_cluster_v4(uint32_t addr, uint32_t rank, float a, float b, float c, float d) {
+    asm volatile(
+        "{\n\t.reg .u32 ra;\n\tmapa.shared::cluster.u32 ra, %0, %1;\n\t"
+        "st.shared::cluster.v4.f32 [ra], {%2, %3, %4, %5};\n\t}" ::"r"(addr),
+        "r"(rank), "f"(a), "f"(b), "f"(c), "f"(d)
+        : "memory");
+}
 
 enum : int { SITE_TC_EMPTY = 21, SITE_TC_FULL = 22, SITE_TC_ACCUM = 23, SITE_TC_DRAIN = 24, SITE_TC_FREE = 25 };
 
@@ -142,15 +171,13 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, float *v) {
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// Epi::pair(t, c, v0, v1): output row t, columns (c, c + 1); Epi::row (when
-// Epi::kRow): the thread's whole span of columns at once, with vector stores
-template <int BN, int WT, class Epi>
+// Epi::row(t, c, v, n): output row t, the thread's span of columns from c on, of
+// which n are inside the matrix
+template <int BN, int SPLIT, int WT, class Epi>
 __global__ void __launch_bounds__(TC_THREADS, 1)
-    gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant__ CUtensorMap map_a1,
-                   const __grid_constant__ CUtensorMap map_a2, const __grid_constant__ CUtensorMap map_w,
-                   const __grid_constant__ CUtensorMap map_w1, const __grid_constant__ CUtensorMap map_w2, int T,
-                   int N, int K, int *err, const Epi epi) {
+    gemm_tc_kernel(const __grid_constant__ GemmMaps maps, int T, int N, int K, int *err, const Epi epi) {
     static_assert(WT == 1 || WT == kTerms, "one exact bf16 weight term, or three");
+    static_assert(SPLIT == 1 || SPLIT == 2 || SPLIT == 4, "CTAs of a tile");
     constexpr int AT = Epi::kATerms;   // activation terms multiplied (and loaded)
     static_assert(AT >= 1 && AT <= kTerms, "activation terms");
     using G = TcTile<BN, AT>;
@@ -165,8 +192,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     const int ntiles = ntm * ntn;
     const int nk = (K + TC_BK - 1) / TC_BK;
     constexpr int WU = WT == 1 ? 1 : Epi::kATerms;  // weight terms used
-    const int nkk = nk * WU;                      // k-blocks of all weight terms
-    const int ngroups = (nkk + TC_GROUP - 1) / TC_GROUP;
+    // this CTA's tiles, and its range of the k-blocks of all weight terms
+    const int rank = (int)blockIdx.x % SPLIT;
+    const int tile0 = (int)blockIdx.x / SPLIT, tile_step = (int)gridDim.x / SPLIT;
+    const int kk_begin = rank * nk * WU / SPLIT, kk_end = (rank + 1) * nk * WU / SPLIT;
+    const int ngroups = (kk_end - kk_begin + TC_GROUP - 1) / TC_GROUP;
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
 
     if (threadIdx.x == 0) {
@@ -196,9 +226,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         if (lane == 0) {  // ------------------------------------------- TMA producer
             int it = 0;   // k-blocks issued over all tiles
             bool ok = true;
-            for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+            for (int tile = tile0; tile < ntiles && ok; tile += tile_step) {
                 const int m0 = (tile % ntm) * TC_BM, n0 = (tile / ntm) * BN;
-                for (int kk = 0; kk < nkk; ++kk, ++it) {
+                const uint32_t a_bytes = (uint32_t)maps.a_rows * (TC_BK * 2);
+                for (int kk = kk_begin; kk < kk_end; ++kk, ++it) {
                     const int s = it % S;
                     if (it >= S && !(ok = mbar_wait(smem_u32(&empty_bar[s]), ((it / S) + 1) & 1, err, SITE_TC_EMPTY)))
                         break;
@@ -207,12 +238,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                     const uint32_t fb = smem_u32(&full_bar[s]);
                     // term j meets the activation terms i <= 2 - j only
                     const int na = AT - j;
-                    mbar_arrive_expect_tx(fb, (uint32_t)na * TC_A_BYTES + G::B_BYTES);
-                    tma_load_2d(st, &map_a0, kb * TC_BK, m0, fb);
-                    if (na > 1) tma_load_2d(st + TC_A_BYTES, &map_a1, kb * TC_BK, m0, fb);
-                    if (na > 2) tma_load_2d(st + 2 * TC_A_BYTES, &map_a2, kb * TC_BK, m0, fb);
-                    tma_load_2d(st + AT * TC_A_BYTES, j == 0 ? &map_w : j == 1 ? &map_w1 : &map_w2, kb * TC_BK, n0,
-                                fb);
+                    mbar_arrive_expect_tx(fb, (uint32_t)na * a_bytes + G::B_BYTES);
+#pragma unroll
+                    for (int t = 0; t < AT; ++t)
+                        if (t < na) tma_load_2d(st + t * TC_A_BYTES, &maps.a[t], kb * TC_BK, m0, fb);
+                    tma_load_2d(st + AT * TC_A_BYTES, &maps.w[j], kb * TC_BK, n0, fb);
                     s_issued = it + 1;
                 }
             }
@@ -222,7 +252,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             constexpr uint32_t idesc = tc_idesc(BN);
             bool ok = true;
             int it = 0, gg = 0;   // k-blocks and groups consumed over all tiles
-            for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+            for (int tile = tile0; tile < ntiles && ok; tile += tile_step) {
                 for (int gi = 0; gi < ngroups && ok; ++gi, ++gg) {
                     const int b = gg & 1;
                     // the epilogue must have read this buffer's previous group
@@ -230,8 +260,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                         break;
                     tc_fence_after();
                     const uint32_t acc = tmem + (uint32_t)b * G::ACC_STRIDE;
-                    const int kk1 = min(nkk, (gi + 1) * TC_GROUP);
-                    for (int kk = gi * TC_GROUP; kk < kk1; ++kk, ++it) {
+                    const int kk0 = kk_begin + gi * TC_GROUP, kk1 = min(kk_end, kk0 + TC_GROUP);
+                    for (int kk = kk0; kk < kk1; ++kk, ++it) {
                         const int s = it % S;
                         ok = mbar_wait(smem_u32(&full_bar[s]), (it / S) & 1, err, SITE_TC_FULL);
                         if (!ok) break;
@@ -247,7 +277,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                             for (int t = 0; t < kTerms; ++t)
                                 if (t < nt)
                                     tc_mma(acc, ad0 + (uint64_t)((t * TC_A_BYTES + 32 * k) >> 4),
-                                           bd0 + (uint64_t)(2 * k), idesc, (kk != gi * TC_GROUP || k != 0 || t != 0));
+                                           bd0 + (uint64_t)(2 * k), idesc, (kk != kk0 || k != 0 || t != 0));
                         tc_commit(smem_u32(&empty_bar[s]));
                     }
                     tc_commit(smem_u32(&acc_full[b]));  // fires when this group's MMAs have completed
@@ -260,7 +290,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
         bool ok = true;
         int gg = 0;
-        for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+        for (int tile = tile0; tile < ntiles && ok; tile += tile_step) {
             const int m0 = (tile % ntm) * TC_BM, n0 = (tile / ntm) * BN;
             const int t = m0 + q * 32 + lane;
             float sum[G::EPI_COLS];
@@ -290,16 +320,50 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&acc_free[b]));
             }
-            if (ok && t < T) {
+            if constexpr (SPLIT == 1) {
                 const int c0 = n0 + half * G::EPI_COLS;
-                if constexpr (Epi::kRow) {
-                    epi.row(t, c0, sum, N - c0);
-                } else {
+                if (ok && t < T) epi.row(t, c0, sum, N - c0);
+            } else {
+                // one tile per CTA: every CTA of the cluster has finished with its ring, so the
+                // sums' column slices cross through it: [source rank][row][SL + 4]
+                constexpr int SL = BN / SPLIT, PITCH = SL + 4;
+                constexpr uint32_t SRC = TC_BM * PITCH * 4;
+                static_assert(SPLIT * SRC <= G::STAGES * G::STAGE_BYTES && SL % 16 == 0, "slices fit the ring");
+                const int row = q * 32 + lane;
+                cluster_sync_all();
 #pragma unroll
-                    for (int j = 0; j < G::EPI_COLS; j += 2)
-                        if (c0 + j < N) epi.pair(t, c0 + j, sum[j], sum[j + 1]);
+                for (int c = 0; c < G::EPI_COLS; c += 4) {
+                    const int col = half * G::EPI_COLS + c;
+                    st_cluster_v4(base + (uint32_t)rank * SRC + (uint32_t)(row * PITCH + col % SL) * 4, col / SL, sum[c],
+                                  sum[c + 1], sum[c + 2], sum[c + 3]);
+                }
+                cluster_sync_all();
+                // this CTA's slice: half of it per warp of a pair, or all of it in the first
+                constexpr int NC = SL % 32 == 0 ? SL / 2 : SL;
+                if (SL % 32 == 0 || half == 0) {
+                    const int part = SL % 32 == 0 ? half * NC : 0;
+                    float v[NC];
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) v[c] = 0.f;
+#pragma unroll
+                    for (int r = 0; r < SPLIT; ++r)
+#pragma unroll
+                        for (int c = 0; c < NC; c += 4) {
+                            const float4 x = *reinterpret_cast<const float4 *>(
+                                smem_raw + (base - smem_u32(smem_raw)) + r * SRC + (size_t)(row * PITCH + part + c) * 4);
+                            v[c] += x.x; v[c + 1] += x.y; v[c + 2] += x.z; v[c + 3] += x.w;
+                        }
+                    const int c0 = n0 + rank * SL + part;
+                    if (ok && t < T && c0 < N) epi.row(t, c0, v, N - c0);
                 }
             }
+        }
+    }
+    if constexpr (SPLIT > 1) {
+        if (warp < 2) {   // the epilogue warps' two cluster barriers count every thread
+            __syncwarp();
+            cluster_sync_all();
+            cluster_sync_all();
         }
     }
     tc_fence_before();

@@ -45,15 +45,21 @@ struct Bufs {
     float *QKraw;
 };
 
-// TMA descriptors of the prefill GEMM operands (built once per context).
-struct PrefillMaps {
-    CUtensorMap a[kTerms], o[kTerms], m[kTerms];       // GEMM activations, 128-row boxes
-    CUtensorMap kv;                                    // the whole KV pool: [page][K|V][kv_head][16][d]
-    std::vector<CUtensorMap> wqkv, wo, wgu, wd;        // per layer weights, boxes of bn_* rows
-    CUtensorMap wt_qkv[kTerms], wt_o[kTerms], wt_gu[kTerms], wt_d[kTerms];  // 8-bit format: the dequantised terms
-    int bn_qkv, bn_o, bn_gu, bn_d;                     // output-tile width of each matrix's GEMM
+// A weight matrix (or one of its terms) as 2-D maps, one per tile width of the GEMM.
+constexpr int kTileWidths = 3;
+constexpr int kTileBn[kTileWidths] = {128, 192, 224};
+struct WeightMaps {
+    CUtensorMap bn[kTileWidths];
 };
 
+// TMA descriptors of the prefill GEMM operands (built once per context).
+struct PrefillMaps {
+    // GEMM activations [i]: boxes of 32 (i + 1) rows, for chunks shorter than a 128-row tile
+    CUtensorMap a[4][kTerms], o[4][kTerms], m[4][kTerms];
+    CUtensorMap kv;                                    // the whole KV pool: [page][K|V][kv_head][16][d]
+    std::vector<WeightMaps> wqkv, wo, wgu, wd;         // per layer weights
+    WeightMaps wt_qkv[kTerms], wt_o[kTerms], wt_gu[kTerms], wt_d[kTerms];  // 8-bit format: the dequantised terms
+};
 
 // A bf16 tensor map with 128-byte swizzle: dims / box / element strides innermost
 // first, strides_bytes[i] the byte stride of dimension i + 1 (false on failure).

@@ -16,25 +16,45 @@
 
 namespace wici {
 
-// output-tile widths of the prefill GEMMs: 128 x 192 tiles (three 72 KB ring
-// stages) or 128 x 128 tiles (three 64 KB stages), chosen per weight matrix
-// for the fewest whole waves of tiles at the largest chunk
-// output-tile width: the fewest columns per SM over the waves of tiles, a
-// 128-column tile charged 10% for reading its A operand more often per FLOP;
-// 224 only for GEMMs of two activation terms (three leave too few ring stages)
-static int pick_bn(int T, int N, int sms, bool allow224) {
-    const int tm = (T + TC_BM - 1) / TC_BM;
-    int best = 0;
+// The tile of one GEMM: its width, and the CTAs that share one (split k-blocks).
+struct TileChoice {
+    int bn, split;
+};
+
+// Chosen per call from the chunk's own length, by modelled SM cycles: waves of tiles x
+// (k-blocks of a CTA x cycles of a k-block + fixed).  A k-block takes its MMAs (bn / 2
+// cycles per 128 x bn x 16 one) or its shared-memory traffic at 115 bytes a cycle (the
+// operands written once, A and B read by every MMA), whichever is longer; measured at
+// 2048 tokens, 8B widths: 1157 cycles for 192 columns and two terms (1214 modelled).
+// fixed is the pipeline's fill and the epilogue, plus the exchange of a split tile.  Split tiles
+// run as one wave only: clusters of two and four CTAs fit 144 and 128 of the 152 SMs.
+// 224 columns only for GEMMs of two activation terms (three leave too few ring stages).
+// The choice used to be made for the largest chunk: a 61-token chunk at 8B widths then
+// ran its O and down projections on 19 CTAs, 41 and 108 us against 26 and 46 now, and a
+// 512-token one at 1B widths took 3731 us instead of 3023.
+static TileChoice pick_tile(int T, int N, int K, int at, int wu, int sms) {
+    const int tm = (T + TC_BM - 1) / TC_BM, nk = (K + TC_BK - 1) / TC_BK * wu;
+    const int rows = T < TC_BM ? (T + 31) / 32 * 32 : TC_BM;
+    const double mmas = wu == 1 ? at : (at + 1) * 0.5;   // per k-block and k-step
+    TileChoice best = {0, 0};
     double best_cost = 0.0;
-    for (int bn : {128, 192, 224}) {
-        if (bn == 224 && !allow224) continue;
-        const int waves = (tm * ((N + bn - 1) / bn) + sms - 1) / sms;
-        const double cost = (double)waves * bn * (bn == 128 ? 1.1 : 1.0);
-        if (best == 0 || cost < best_cost) {
-            best = bn;
-            best_cost = cost;
+    for (int bn : kTileBn)
+        for (int split : {1, 2, 4}) {
+            if (bn == 224 && (at != 2 || split != 1)) continue;
+            const int units = tm * ((N + bn - 1) / bn) * split;
+            if (split > 1 && units > (split == 2 ? sms * 144 / 152 : sms * 128 / 152)) continue;
+            const double mma = 2.0 * bn * mmas;
+            // 192 columns and three terms leave three ring stages: 8% more per k-block than the ports ask for
+            const double smem = ((mmas * rows + bn) * 128.0 + 4.0 * mmas * (4096.0 + 32.0 * bn)) /
+                                (at == 3 && bn == 192 ? 106.0 : 115.0);
+            const double cost = (double)((units + sms - 1) / sms) *
+                                ((double)((nk + split - 1) / split) * (mma > smem ? mma : smem) + 2500.0 +
+                                 (split > 1 ? 2500.0 : 0.0));
+            if (best.bn == 0 || cost < best_cost) {
+                best = {bn, split};
+                best_cost = cost;
+            }
         }
-    }
     return best;
 }
 
@@ -461,6 +481,12 @@ static bool encode_2d(CUtensorMap *m, const void *ptr, int rows, int K, int box_
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+static bool encode_w(WeightMaps *m, const void *ptr, int rows, int K) {
+    bool ok = true;
+    for (int i = 0; i < kTileWidths; ++i) ok = ok && encode_2d(&m->bn[i], ptr, rows, K, kTileBn[i]);
+    return ok;
+}
+
 // the KV pool of every layer as [page (layer-major)][K|V][kv head][16 slots][d]:
 // boxes of 64 d x 16 slots of one (page, K|V, head)
 static bool encode_kv(CUtensorMap *m, const void *ptr, const Plan &p) {
@@ -481,22 +507,19 @@ const char *make_prefill_maps(const Plan &p, const Bufs &b, PrefillMaps *m) {
     const int T = p.max_chunk;
     bool ok = true;
     for (int t = 0; t < kTerms; ++t)
-        ok = ok && encode_2d(&m->a[t], b.A[t], T, p.H, TC_BM) && encode_2d(&m->o[t], b.O[t], T, p.qdim, TC_BM) &&
-             encode_2d(&m->m[t], b.M[t], T, p.F, TC_BM);
+        for (int x = 0; x < 4; ++x) {
+            const int box = 32 * (x + 1);
+            ok = ok && encode_2d(&m->a[x][t], b.A[t], T, p.H, box) && encode_2d(&m->o[x][t], b.O[t], T, p.qdim, box) &&
+                 encode_2d(&m->m[x][t], b.M[t], T, p.F, box);
+        }
     if (!ok) return "cuTensorMapEncodeTiled failed for an activation operand";
     ok = encode_kv(&m->kv, b.KV, p);
     if (!ok) return "cuTensorMapEncodeTiled failed for the attention operands";
-    m->bn_qkv = pick_bn(T, p.nqkv, p.num_sms, PEpiQKV::kATerms == 2);
-    m->bn_o = pick_bn(T, p.H, p.num_sms, PEpiResidual::kATerms == 2);
-    m->bn_gu = pick_bn(T, 2 * p.F, p.num_sms, PEpiSwiGLU::kATerms == 2);
-    m->bn_d = pick_bn(T, p.H, p.num_sms, PEpiResidual::kATerms == 2);
     if (p.q8) {
         // the 8-bit format: every GEMM reads the one dequantised matrix in the workspace
         for (int t = 0; t < kTerms; ++t) {
-            ok = encode_2d(&m->wt_qkv[t], b.Wt[t], p.nqkv, p.H, m->bn_qkv) &&
-                 encode_2d(&m->wt_o[t], b.Wt[t], p.H, p.qdim, m->bn_o) &&
-                 encode_2d(&m->wt_gu[t], b.Wt[t], 2 * p.F, p.H, m->bn_gu) &&
-                 encode_2d(&m->wt_d[t], b.Wt[t], p.H, p.F, m->bn_d);
+            ok = encode_w(&m->wt_qkv[t], b.Wt[t], p.nqkv, p.H) && encode_w(&m->wt_o[t], b.Wt[t], p.H, p.qdim) &&
+                 encode_w(&m->wt_gu[t], b.Wt[t], 2 * p.F, p.H) && encode_w(&m->wt_d[t], b.Wt[t], p.H, p.F);
             if (!ok) return "cuTensorMapEncodeTiled failed for a dequantised weight matrix";
         }
     }
@@ -506,10 +529,8 @@ const char *make_prefill_maps(const Plan &p, const Bufs &b, PrefillMaps *m) {
     m->wd.resize(p.q8 ? 0 : p.L);
     for (int l = 0; l < (p.q8 ? 0 : p.L); ++l) {
         const LayerOffsets &lo = p.layer[l];
-        ok = encode_2d(&m->wqkv[l], b.W + lo.wqkv, p.nqkv, p.H, m->bn_qkv) &&
-             encode_2d(&m->wo[l], b.W + lo.wo, p.H, p.qdim, m->bn_o) &&
-             encode_2d(&m->wgu[l], b.W + lo.wgu, 2 * p.F, p.H, m->bn_gu) &&
-             encode_2d(&m->wd[l], b.W + lo.wd, p.H, p.F, m->bn_d);
+        ok = encode_w(&m->wqkv[l], b.W + lo.wqkv, p.nqkv, p.H) && encode_w(&m->wo[l], b.W + lo.wo, p.H, p.qdim) &&
+             encode_w(&m->wgu[l], b.W + lo.wgu, 2 * p.F, p.H) && encode_w(&m->wd[l], b.W + lo.wd, p.H, p.F);
         if (!ok) return "cuTensorMapEncodeTiled failed for a weight matrix";
     }
     static bool attrs = false;
@@ -517,21 +538,24 @@ const char *make_prefill_maps(const Plan &p, const Bufs &b, PrefillMaps *m) {
         const auto attr = [](const void *f, int bytes) {
             return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
         };
-#define WICI_GEMM_ATTR(BN, WT, E) attr((const void *)gemm_tc_kernel<BN, WT, E>, (int)TcTile<BN, E::kATerms>::SMEM)
-        if (!WICI_GEMM_ATTR(192, 1, PEpiQKV) || !WICI_GEMM_ATTR(192, 1, PEpiResidual) ||
-            !WICI_GEMM_ATTR(192, 1, PEpiSwiGLU) || !WICI_GEMM_ATTR(128, 1, PEpiQKV) ||
-            !WICI_GEMM_ATTR(128, 1, PEpiResidual) || !WICI_GEMM_ATTR(128, 1, PEpiSwiGLU) ||
-            !WICI_GEMM_ATTR(192, kTerms, PEpiQKV) || !WICI_GEMM_ATTR(192, kTerms, PEpiResidual) ||
-            !WICI_GEMM_ATTR(192, kTerms, PEpiSwiGLU) || !WICI_GEMM_ATTR(128, kTerms, PEpiQKV) ||
-            !WICI_GEMM_ATTR(128, kTerms, PEpiResidual) || !WICI_GEMM_ATTR(128, kTerms, PEpiSwiGLU) ||
-            !WICI_GEMM_ATTR(224, 1, PEpiResidual) || !WICI_GEMM_ATTR(224, 1, PEpiSwiGLU) ||
-            !WICI_GEMM_ATTR(224, kTerms, PEpiResidual) || !WICI_GEMM_ATTR(224, kTerms, PEpiSwiGLU) ||
+        bool set = true;
+#define WICI_GEMM_ATTR(BN, SPLIT, WT, E) \
+    set = set && attr((const void *)gemm_tc_kernel<BN, SPLIT, WT, E>, (int)TcTile<BN, E::kATerms>::SMEM);
+#define WICI_GEMM_ATTRS(WT, E)                                                                              \
+    WICI_GEMM_ATTR(128, 1, WT, E) WICI_GEMM_ATTR(128, 2, WT, E) WICI_GEMM_ATTR(128, 4, WT, E)              \
+    WICI_GEMM_ATTR(192, 1, WT, E) WICI_GEMM_ATTR(192, 2, WT, E) WICI_GEMM_ATTR(192, 4, WT, E)
+        WICI_GEMM_ATTRS(1, PEpiQKV) WICI_GEMM_ATTRS(1, PEpiResidual) WICI_GEMM_ATTRS(1, PEpiSwiGLU)
+        WICI_GEMM_ATTRS(kTerms, PEpiQKV) WICI_GEMM_ATTRS(kTerms, PEpiResidual) WICI_GEMM_ATTRS(kTerms, PEpiSwiGLU)
+        WICI_GEMM_ATTR(224, 1, 1, PEpiResidual) WICI_GEMM_ATTR(224, 1, 1, PEpiSwiGLU)
+        WICI_GEMM_ATTR(224, 1, kTerms, PEpiResidual) WICI_GEMM_ATTR(224, 1, kTerms, PEpiSwiGLU)
+#undef WICI_GEMM_ATTRS
+#undef WICI_GEMM_ATTR
+        if (!set ||
             cudaFuncSetAttribute(attn_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)(AttnSmem<128>::TOTAL + 1024)) != cudaSuccess ||
             cudaFuncSetAttribute(attn_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)(AttnSmem<64>::TOTAL + 1024)) != cudaSuccess)
             return "cannot raise the shared-memory limit of the tensor-core GEMM";
-#undef WICI_GEMM_ATTR
         attrs = true;
     }
     return nullptr;
@@ -563,44 +587,67 @@ cudaError_t launch_attn_tc(const Plan &p, const Bufs &b, const PrefillMaps &mp, 
 
 // the weight operand of one GEMM: one exact bf16 matrix, or three terms
 struct WOperand {
-    const CUtensorMap *w[kTerms];
+    const WeightMaps *w[kTerms];
     int terms;
 };
 
-template <int BN, class Epi>
-static void launch_gemm(const Plan &p, const CUtensorMap *a, const WOperand &w, int T, int N, int K, int *err,
-                        const Epi &epi, cudaStream_t st) {
+template <int BN, int SPLIT, class Epi>
+static cudaError_t launch_gemm(const Plan &p, const GemmMaps &maps, int terms, int T, int N, int K, int *err,
+                               const Epi &epi, cudaStream_t st) {
     const int tiles = ((T + TC_BM - 1) / TC_BM) * ((N + BN - 1) / BN);
-    const int grid = tiles < p.num_sms ? tiles : p.num_sms;   // persistent: at most one CTA per SM
-    if (w.terms == 1)
-        gemm_tc_kernel<BN, 1, Epi><<<grid, TC_THREADS, TcTile<BN, Epi::kATerms>::SMEM, st>>>(a[0], a[1], a[2], *w.w[0], *w.w[1],
-                                                                              *w.w[2], T, N, K, err, epi);
-    else
-        gemm_tc_kernel<BN, kTerms, Epi><<<grid, TC_THREADS, TcTile<BN, Epi::kATerms>::SMEM, st>>>(
-            a[0], a[1], a[2], *w.w[0], *w.w[1], *w.w[2], T, N, K, err, epi);
+    cudaLaunchConfig_t cfg = {};
+    // persistent, at most one CTA per SM; a split tile's CTAs are one cluster
+    cfg.gridDim = dim3(SPLIT > 1 ? tiles * SPLIT : tiles < p.num_sms ? tiles : p.num_sms);
+    cfg.blockDim = dim3(TC_THREADS);
+    cfg.dynamicSmemBytes = TcTile<BN, Epi::kATerms>::SMEM;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = SPLIT;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = SPLIT > 1 ? 1 : 0;
+    if (terms == 1) return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<BN, SPLIT, 1, Epi>, maps, T, N, K, err, epi);
+    return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<BN, SPLIT, kTerms, Epi>, maps, T, N, K, err, epi);
 }
 
+// a: the activation's maps with boxes of 32, 64, 96 and 128 rows
 template <class Epi>
-static cudaError_t gemm(const Plan &p, int bn, const CUtensorMap *a, const WOperand &w, int T, int N, int K,
+static cudaError_t gemm(const Plan &p, const CUtensorMap (&a)[4][kTerms], const WOperand &w, int T, int N, int K,
                         int *err, const Epi &epi, cudaStream_t st, LaunchHook *hook, const char *name) {
+    const TileChoice c = pick_tile(T, N, K, Epi::kATerms, w.terms == 1 ? 1 : Epi::kATerms, p.num_sms);
+    GemmMaps maps;
+    const int box = T < TC_BM ? (T - 1) / 32 : 3;   // rows of a tile past the chunk are not loaded
+    maps.a_rows = 32 * (box + 1);
+    for (int t = 0; t < kTerms; ++t) {
+        maps.a[t] = a[box][t];
+        for (int i = 0; i < kTileWidths; ++i)
+            if (kTileBn[i] == c.bn) maps.w[t] = w.w[t]->bn[i];
+    }
     if (hook) hook->before(name);
-    if (bn == 128)
-        launch_gemm<128>(p, a, w, T, N, K, err, epi, st);
-    else if (bn == 192)
-        launch_gemm<192>(p, a, w, T, N, K, err, epi, st);
+    cudaError_t e;
+    if (c.bn == 128)
+        e = c.split == 1   ? launch_gemm<128, 1>(p, maps, w.terms, T, N, K, err, epi, st)
+            : c.split == 2 ? launch_gemm<128, 2>(p, maps, w.terms, T, N, K, err, epi, st)
+                           : launch_gemm<128, 4>(p, maps, w.terms, T, N, K, err, epi, st);
+    else if (c.bn == 192)
+        e = c.split == 1   ? launch_gemm<192, 1>(p, maps, w.terms, T, N, K, err, epi, st)
+            : c.split == 2 ? launch_gemm<192, 2>(p, maps, w.terms, T, N, K, err, epi, st)
+                           : launch_gemm<192, 4>(p, maps, w.terms, T, N, K, err, epi, st);
     else if constexpr (Epi::kATerms == 2)
-        launch_gemm<224>(p, a, w, T, N, K, err, epi, st);
+        e = launch_gemm<224, 1>(p, maps, w.terms, T, N, K, err, epi, st);
     else
-        return cudaErrorInvalidValue;   // pick_bn never picks 224 for three terms
+        e = cudaErrorInvalidValue;   // pick_tile never picks 224 for three terms
     if (hook) hook->after(name);
-    return cudaGetLastError();
+    return e;
 }
 
 // bf16: the layer's own matrix; 8-bit format: dequantise the layer's rows into
 // the workspace terms first (stream order makes the previous GEMM finish reading them)
 template <class Epi>
-static cudaError_t weight_operand(const Plan &p, const Bufs &b, const CUtensorMap &bf16_map,
-                                  const CUtensorMap *terms, const uint16_t *rows, int n_rows, int K, cudaStream_t st,
+static cudaError_t weight_operand(const Plan &p, const Bufs &b, const WeightMaps &bf16_map,
+                                  const WeightMaps *terms, const uint16_t *rows, int n_rows, int K, cudaStream_t st,
                                   LaunchHook *hook, WOperand *w) {
     if (!p.q8) {
         *w = WOperand{{&bf16_map, &bf16_map, &bf16_map}, 1};
@@ -628,7 +675,7 @@ cudaError_t enqueue_prefill_chunk(const Plan &p, const Bufs &b, const PrefillMap
         if ((e = weight_operand<PEpiQKV>(p, b, p.q8 ? mp.wt_qkv[0] : mp.wqkv[l], mp.wt_qkv, b.W + lo.wqkv, p.nqkv, p.H, st,
                                 hook, &w)) != cudaSuccess)
             return e;
-        if ((e = gemm(p, mp.bn_qkv, mp.a, w, T, p.nqkv, p.H, err, eq, st, hook, "prefill_qkv")) != cudaSuccess)
+        if ((e = gemm(p, mp.a, w, T, p.nqkv, p.H, err, eq, st, hook, "prefill_qkv")) != cudaSuccess)
             return e;
         if (p.qk_norm) {
             // Qwen3 block: per-head q/k norm, then RoPE and the operand / page stores
@@ -653,7 +700,7 @@ cudaError_t enqueue_prefill_chunk(const Plan &p, const Bufs &b, const PrefillMap
         if ((e = weight_operand<PEpiResidual>(p, b, p.q8 ? mp.wt_o[0] : mp.wo[l], mp.wt_o, b.W + lo.wo, p.H, p.qdim, st, hook,
                                 &w)) != cudaSuccess)
             return e;
-        if ((e = gemm(p, mp.bn_o, mp.o, w, T, p.H, p.qdim, err, PEpiResidual{b.X, p.H}, st, hook,
+        if ((e = gemm(p, mp.o, w, T, p.H, p.qdim, err, PEpiResidual{b.X, p.H}, st, hook,
                       "prefill_o_proj")) != cudaSuccess)
             return e;
         // A7: RMSNorm + gate/up + SwiGLU
@@ -662,14 +709,14 @@ cudaError_t enqueue_prefill_chunk(const Plan &p, const Bufs &b, const PrefillMap
         if ((e = weight_operand<PEpiSwiGLU>(p, b, p.q8 ? mp.wt_gu[0] : mp.wgu[l], mp.wt_gu, b.W + lo.wgu, 2 * p.F, p.H, st,
                                 hook, &w)) != cudaSuccess)
             return e;
-        if ((e = gemm(p, mp.bn_gu, mp.a, w, T, 2 * p.F, p.H, err, PEpiSwiGLU{M, p.F}, st, hook,
+        if ((e = gemm(p, mp.a, w, T, 2 * p.F, p.H, err, PEpiSwiGLU{M, p.F}, st, hook,
                       "prefill_gate_up")) != cudaSuccess)
             return e;
         // A8: down projection + residual
         if ((e = weight_operand<PEpiResidual>(p, b, p.q8 ? mp.wt_d[0] : mp.wd[l], mp.wt_d, b.W + lo.wd, p.H, p.F, st, hook,
                                 &w)) != cudaSuccess)
             return e;
-        if ((e = gemm(p, mp.bn_d, mp.m, w, T, p.H, p.F, err, PEpiResidual{b.X, p.H}, st, hook,
+        if ((e = gemm(p, mp.m, w, T, p.H, p.F, err, PEpiResidual{b.X, p.H}, st, hook,
                       "prefill_down")) != cudaSuccess)
             return e;
     }
