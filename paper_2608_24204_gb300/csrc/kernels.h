@@ -45,11 +45,12 @@ struct Bufs {
     float *QKraw;
 };
 
-// A weight matrix (or one of its terms) as 2-D maps, one per tile width of the GEMM.
-constexpr int kTileWidths = 3;
-constexpr int kTileBn[kTileWidths] = {128, 192, 224};
+// A weight matrix (or one of its terms) as 2-D maps with the boxes of the GEMM's tiles:
+// the tile's columns, or half of them where a pair of CTAs shares it.
+constexpr int kWeightBoxes = 5;
+constexpr int kWeightBox[kWeightBoxes] = {96, 112, 128, 192, 224};
 struct WeightMaps {
-    CUtensorMap bn[kTileWidths];
+    CUtensorMap box[kWeightBoxes];
 };
 
 // TMA descriptors of the prefill GEMM operands (built once per context).
@@ -59,6 +60,7 @@ struct PrefillMaps {
     CUtensorMap kv;                                    // the whole KV pool: [page][K|V][kv_head][16][d]
     std::vector<WeightMaps> wqkv, wo, wgu, wd;         // per layer weights
     WeightMaps wt_qkv[kTerms], wt_o[kTerms], wt_gu[kTerms], wt_d[kTerms];  // 8-bit format: the dequantised terms
+    int sms, pairs, quads;   // CTAs, clusters of two and clusters of four that run at once
 };
 
 // A bf16 tensor map with 128-byte swizzle: dims / box / element strides innermost

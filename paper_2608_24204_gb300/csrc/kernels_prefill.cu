@@ -11,50 +11,60 @@
 
 #include "common.cuh"
 #include "attn_tc.cuh"
+#include "gemm2_tc.cuh"
 #include "gemm_tc.cuh"
 #include "kernels.h"
 
 namespace wici {
 
-// The tile of one GEMM: its width, and the CTAs that share one (split k-blocks).
+// The tile of one GEMM: its width, the CTAs that share one by splitting the k-blocks, or
+// a pair of CTAs on a tile of 256 rows.
 struct TileChoice {
     int bn, split;
+    bool pair;
 };
 
 // Chosen per call from the chunk's own length, by modelled SM cycles: waves of tiles x
 // (k-blocks of a CTA x cycles of a k-block + fixed).  A k-block takes its MMAs (bn / 2
-// cycles per 128 x bn x 16 one) or its shared-memory traffic at 115 bytes a cycle (the
-// operands written once, A and B read by every MMA), whichever is longer; measured at
-// 2048 tokens, 8B widths: 1157 cycles for 192 columns and two terms (1214 modelled).
-// fixed is the pipeline's fill and the epilogue, plus the exchange of a split tile.  Split tiles
-// run as one wave only: clusters of two and four CTAs fit 144 and 128 of the 152 SMs.
-// 224 columns only for GEMMs of two activation terms (three leave too few ring stages).
+// cycles per 128 (256 for a pair) x bn x 16 one) or its shared-memory traffic at 115 bytes
+// a cycle (the operands written once, A and B read by every MMA; half of B per CTA of a
+// pair), whichever is longer; measured at 2048 tokens, 8B widths: 1157 cycles for 192
+// columns and two terms (1214 modelled).  fixed is the pipeline's fill and the epilogue,
+// plus the exchange of a split tile.  Split tiles run as one wave only; how many clusters
+// fit at once the driver says (SMs come in groups that they may not divide).  224 columns without a pair only for
+// GEMMs of two activation terms (three leave too few ring stages).
 // The choice used to be made for the largest chunk: a 61-token chunk at 8B widths then
 // ran its O and down projections on 19 CTAs, 41 and 108 us against 26 and 46 now, and a
 // 512-token one at 1B widths took 3731 us instead of 3023.
-static TileChoice pick_tile(int T, int N, int K, int at, int wu, int sms) {
-    const int tm = (T + TC_BM - 1) / TC_BM, nk = (K + TC_BK - 1) / TC_BK * wu;
-    const int rows = T < TC_BM ? (T + 31) / 32 * 32 : TC_BM;
+static TileChoice pick_tile(int T, int N, int K, int at, int wu, const PrefillMaps &mp) {
+    const int nk = (K + TC_BK - 1) / TC_BK * wu;
     const double mmas = wu == 1 ? at : (at + 1) * 0.5;   // per k-block and k-step
-    TileChoice best = {0, 0};
+    TileChoice best = {0, 0, false};
     double best_cost = 0.0;
-    for (int bn : kTileBn)
+    auto consider = [&](TileChoice c, int units, int slots, double rows, double b_rows, double port) {
+        const double mma = 2.0 * c.bn * mmas;
+        const double smem = ((mmas * rows + b_rows) * 128.0 + 4.0 * mmas * (4096.0 + 32.0 * b_rows)) / port;
+        const double cost = (double)((units + slots - 1) / slots) *
+                            ((double)((nk + c.split - 1) / c.split) * (mma > smem ? mma : smem) + 2500.0 +
+                             (c.split > 1 ? 2500.0 : 0.0));
+        if (best.bn == 0 || cost < best_cost) {
+            best = c;
+            best_cost = cost;
+        }
+    };
+    const int tm = (T + TC_BM - 1) / TC_BM, tm2 = (T + 2 * TC_BM - 1) / (2 * TC_BM);
+    const int rows = T < TC_BM ? (T + 31) / 32 * 32 : TC_BM;
+    for (int bn : {128, 192, 224})
         for (int split : {1, 2, 4}) {
             if (bn == 224 && (at != 2 || split != 1)) continue;
             const int units = tm * ((N + bn - 1) / bn) * split;
-            if (split > 1 && units > (split == 2 ? sms * 144 / 152 : sms * 128 / 152)) continue;
-            const double mma = 2.0 * bn * mmas;
+            if (split > 1 && units > (split == 2 ? 2 * mp.pairs : 4 * mp.quads)) continue;
             // 192 columns and three terms leave three ring stages: 8% more per k-block than the ports ask for
-            const double smem = ((mmas * rows + bn) * 128.0 + 4.0 * mmas * (4096.0 + 32.0 * bn)) /
-                                (at == 3 && bn == 192 ? 106.0 : 115.0);
-            const double cost = (double)((units + sms - 1) / sms) *
-                                ((double)((nk + split - 1) / split) * (mma > smem ? mma : smem) + 2500.0 +
-                                 (split > 1 ? 2500.0 : 0.0));
-            if (best.bn == 0 || cost < best_cost) {
-                best = {bn, split};
-                best_cost = cost;
-            }
+            consider({bn, split, false}, units, mp.sms, rows, bn, at == 3 && bn == 192 ? 106.0 : 115.0);
         }
+    if (T > TC_BM && mp.pairs > 0)
+        for (int bn : {192, 224, 256})
+            consider({bn, 1, true}, tm2 * ((N + bn - 1) / bn), mp.pairs, TC_BM, bn / 2, 115.0);
     return best;
 }
 
@@ -483,7 +493,7 @@ static bool encode_2d(CUtensorMap *m, const void *ptr, int rows, int K, int box_
 
 static bool encode_w(WeightMaps *m, const void *ptr, int rows, int K) {
     bool ok = true;
-    for (int i = 0; i < kTileWidths; ++i) ok = ok && encode_2d(&m->bn[i], ptr, rows, K, kTileBn[i]);
+    for (int i = 0; i < kWeightBoxes; ++i) ok = ok && encode_2d(&m->box[i], ptr, rows, K, kWeightBox[i]);
     return ok;
 }
 
@@ -548,6 +558,13 @@ const char *make_prefill_maps(const Plan &p, const Bufs &b, PrefillMaps *m) {
         WICI_GEMM_ATTRS(kTerms, PEpiQKV) WICI_GEMM_ATTRS(kTerms, PEpiResidual) WICI_GEMM_ATTRS(kTerms, PEpiSwiGLU)
         WICI_GEMM_ATTR(224, 1, 1, PEpiResidual) WICI_GEMM_ATTR(224, 1, 1, PEpiSwiGLU)
         WICI_GEMM_ATTR(224, 1, kTerms, PEpiResidual) WICI_GEMM_ATTR(224, 1, kTerms, PEpiSwiGLU)
+#define WICI_GEMM2_ATTR(BN, WT, E) \
+    set = set && attr((const void *)gemm2_tc_kernel<BN, WT, E>, (int)TcPairTile<BN, E::kATerms>::SMEM);
+#define WICI_GEMM2_ATTRS(WT, E) WICI_GEMM2_ATTR(192, WT, E) WICI_GEMM2_ATTR(224, WT, E) WICI_GEMM2_ATTR(256, WT, E)
+        WICI_GEMM2_ATTRS(1, PEpiQKV) WICI_GEMM2_ATTRS(1, PEpiResidual) WICI_GEMM2_ATTRS(1, PEpiSwiGLU)
+        WICI_GEMM2_ATTRS(kTerms, PEpiQKV) WICI_GEMM2_ATTRS(kTerms, PEpiResidual) WICI_GEMM2_ATTRS(kTerms, PEpiSwiGLU)
+#undef WICI_GEMM2_ATTRS
+#undef WICI_GEMM2_ATTR
 #undef WICI_GEMM_ATTRS
 #undef WICI_GEMM_ATTR
         if (!set ||
@@ -557,6 +574,32 @@ const char *make_prefill_maps(const Plan &p, const Bufs &b, PrefillMaps *m) {
                                  (int)(AttnSmem<64>::TOTAL + 1024)) != cudaSuccess)
             return "cannot raise the shared-memory limit of the tensor-core GEMM";
         attrs = true;
+    }
+    // resident clusters of two (the pair kernel) and of four, within this context's SM share
+    m->sms = p.num_sms;
+    for (int size : {2, 4}) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(size * p.num_sms));
+        cfg.blockDim = dim3(TC_THREADS);
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = size;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        cudaError_t e;
+        if (size == 2) {
+            cfg.dynamicSmemBytes = TcPairTile<256, 2>::SMEM;
+            e = cudaOccupancyMaxActiveClusters(&n, gemm2_tc_kernel<256, 1, PEpiSwiGLU>, &cfg);
+        } else {
+            cfg.dynamicSmemBytes = TcTile<128, 2>::SMEM;
+            e = cudaOccupancyMaxActiveClusters(&n, gemm_tc_kernel<128, 4, 1, PEpiSwiGLU>, &cfg);
+        }
+        if (e != cudaSuccess) return "cannot query the resident clusters of the tensor-core GEMM";
+        n = n < p.num_sms / size ? n : p.num_sms / size;
+        (size == 2 ? m->pairs : m->quads) = n;
     }
     return nullptr;
 }
@@ -612,22 +655,40 @@ static cudaError_t launch_gemm(const Plan &p, const GemmMaps &maps, int terms, i
     return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<BN, SPLIT, kTerms, Epi>, maps, T, N, K, err, epi);
 }
 
+template <int BN, class Epi>
+static cudaError_t launch_gemm_pair(int pairs, const GemmMaps &maps, int terms, int T, int N, int K, int *err,
+                                    const Epi &epi, cudaStream_t st) {
+    const int tiles = ((T + 2 * TC_BM - 1) / (2 * TC_BM)) * ((N + BN - 1) / BN);
+    const int grid = 2 * (tiles < pairs ? tiles : pairs);
+    constexpr size_t smem = TcPairTile<BN, Epi::kATerms>::SMEM;
+    if (terms == 1)
+        gemm2_tc_kernel<BN, 1, Epi><<<grid, TC_THREADS, smem, st>>>(maps, T, N, K, err, epi);
+    else
+        gemm2_tc_kernel<BN, kTerms, Epi><<<grid, TC_THREADS, smem, st>>>(maps, T, N, K, err, epi);
+    return cudaGetLastError();
+}
+
 // a: the activation's maps with boxes of 32, 64, 96 and 128 rows
 template <class Epi>
-static cudaError_t gemm(const Plan &p, const CUtensorMap (&a)[4][kTerms], const WOperand &w, int T, int N, int K,
-                        int *err, const Epi &epi, cudaStream_t st, LaunchHook *hook, const char *name) {
-    const TileChoice c = pick_tile(T, N, K, Epi::kATerms, w.terms == 1 ? 1 : Epi::kATerms, p.num_sms);
+static cudaError_t gemm(const Plan &p, const PrefillMaps &mp, const CUtensorMap (&a)[4][kTerms], const WOperand &w,
+                        int T, int N, int K, int *err, const Epi &epi, cudaStream_t st, LaunchHook *hook,
+                        const char *name) {
+    const TileChoice c = pick_tile(T, N, K, Epi::kATerms, w.terms == 1 ? 1 : Epi::kATerms, mp);
     GemmMaps maps;
     const int box = T < TC_BM ? (T - 1) / 32 : 3;   // rows of a tile past the chunk are not loaded
     maps.a_rows = 32 * (box + 1);
     for (int t = 0; t < kTerms; ++t) {
         maps.a[t] = a[box][t];
-        for (int i = 0; i < kTileWidths; ++i)
-            if (kTileBn[i] == c.bn) maps.w[t] = w.w[t]->bn[i];
+        for (int i = 0; i < kWeightBoxes; ++i)
+            if (kWeightBox[i] == (c.pair ? c.bn / 2 : c.bn)) maps.w[t] = w.w[t]->box[i];
     }
     if (hook) hook->before(name);
     cudaError_t e;
-    if (c.bn == 128)
+    if (c.pair)
+        e = c.bn == 256   ? launch_gemm_pair<256>(mp.pairs, maps, w.terms, T, N, K, err, epi, st)
+            : c.bn == 224 ? launch_gemm_pair<224>(mp.pairs, maps, w.terms, T, N, K, err, epi, st)
+                          : launch_gemm_pair<192>(mp.pairs, maps, w.terms, T, N, K, err, epi, st);
+    else if (c.bn == 128)
         e = c.split == 1   ? launch_gemm<128, 1>(p, maps, w.terms, T, N, K, err, epi, st)
             : c.split == 2 ? launch_gemm<128, 2>(p, maps, w.terms, T, N, K, err, epi, st)
                            : launch_gemm<128, 4>(p, maps, w.terms, T, N, K, err, epi, st);
@@ -675,7 +736,7 @@ cudaError_t enqueue_prefill_chunk(const Plan &p, const Bufs &b, const PrefillMap
         if ((e = weight_operand<PEpiQKV>(p, b, p.q8 ? mp.wt_qkv[0] : mp.wqkv[l], mp.wt_qkv, b.W + lo.wqkv, p.nqkv, p.H, st,
                                 hook, &w)) != cudaSuccess)
             return e;
-        if ((e = gemm(p, mp.a, w, T, p.nqkv, p.H, err, eq, st, hook, "prefill_qkv")) != cudaSuccess)
+        if ((e = gemm(p, mp, mp.a, w, T, p.nqkv, p.H, err, eq, st, hook, "prefill_qkv")) != cudaSuccess)
             return e;
         if (p.qk_norm) {
             // Qwen3 block: per-head q/k norm, then RoPE and the operand / page stores
@@ -700,7 +761,7 @@ cudaError_t enqueue_prefill_chunk(const Plan &p, const Bufs &b, const PrefillMap
         if ((e = weight_operand<PEpiResidual>(p, b, p.q8 ? mp.wt_o[0] : mp.wo[l], mp.wt_o, b.W + lo.wo, p.H, p.qdim, st, hook,
                                 &w)) != cudaSuccess)
             return e;
-        if ((e = gemm(p, mp.o, w, T, p.H, p.qdim, err, PEpiResidual{b.X, p.H}, st, hook,
+        if ((e = gemm(p, mp, mp.o, w, T, p.H, p.qdim, err, PEpiResidual{b.X, p.H}, st, hook,
                       "prefill_o_proj")) != cudaSuccess)
             return e;
         // A7: RMSNorm + gate/up + SwiGLU
@@ -709,14 +770,14 @@ cudaError_t enqueue_prefill_chunk(const Plan &p, const Bufs &b, const PrefillMap
         if ((e = weight_operand<PEpiSwiGLU>(p, b, p.q8 ? mp.wt_gu[0] : mp.wgu[l], mp.wt_gu, b.W + lo.wgu, 2 * p.F, p.H, st,
                                 hook, &w)) != cudaSuccess)
             return e;
-        if ((e = gemm(p, mp.a, w, T, 2 * p.F, p.H, err, PEpiSwiGLU{M, p.F}, st, hook,
+        if ((e = gemm(p, mp, mp.a, w, T, 2 * p.F, p.H, err, PEpiSwiGLU{M, p.F}, st, hook,
                       "prefill_gate_up")) != cudaSuccess)
             return e;
         // A8: down projection + residual
         if ((e = weight_operand<PEpiResidual>(p, b, p.q8 ? mp.wt_d[0] : mp.wd[l], mp.wt_d, b.W + lo.wd, p.H, p.F, st, hook,
                                 &w)) != cudaSuccess)
             return e;
-        if ((e = gemm(p, mp.m, w, T, p.H, p.F, err, PEpiResidual{b.X, p.H}, st, hook,
+        if ((e = gemm(p, mp, mp.m, w, T, p.H, p.F, err, PEpiResidual{b.X, p.H}, st, hook,
                       "prefill_down")) != cudaSuccess)
             return e;
     }

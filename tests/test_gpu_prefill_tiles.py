@@ -1,6 +1,6 @@
 """Prefill GEMMs over the tile shapes their rule picks for short and ragged chunks:
-tiles shared by two and four CTAs, activation boxes of 32 rows (chunks up to 96
-tokens), a chunk that ends one token into a tile, and widths whose last tile is
+tiles shared by two and four CTAs, activation boxes of 32 to 96 rows, pairs of CTAs on
+256-row tiles, a chunk that ends one token into a tile, and widths whose last tile is
 partly outside the matrix.  Against the fp64 oracle with the parity rules."""
 import pytest
 
@@ -32,8 +32,13 @@ RAGGED = gen.TINY.with_(name="ragged", hidden=512, n_q_heads=12, n_kv_heads=4, f
     (W8B, 61, 2048, True),
     (W1B, 40, 2048, False),
     (W1B, 300, 2048, False),
+    (W8B, 257, 2048, False),     # pairs of CTAs: a second 256-row tile of one row
+    (W8B, 640, 2048, False),
+    (W1B, 1100, 2048, False),
+    (W8B, 300, 2048, True),
     (RAGGED, 50, 2048, False),
     (RAGGED, 200, 2048, False),
+    (RAGGED, 1500, 2048, False),
 ])
 def test_prefill_tile_choices(cfg, prompt, chunk, q8):
     cfg = cfg.with_(prompt_len=prompt, decode_steps=1)
