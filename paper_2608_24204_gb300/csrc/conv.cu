@@ -8,6 +8,7 @@
 #include <mutex>
 
 #include "../../include/wici.h"
+#include "conv2_tc.cuh"
 #include "conv_tc.cuh"
 #include "kernels.h"
 
@@ -39,23 +40,59 @@ bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
 std::mutex g_mu;
 int g_attr_device = -1;
+int g_sms = 0, g_clusters[4] = {};   // SMs; resident clusters of 1, 2, 4 and 8 CTAs
 
-cudaError_t setup(int *nsm) {
+template <int MODE>
+cudaError_t setup_mode() {
+    cudaError_t e = cudaSuccess;
+    for (const void *f : {(const void *)conv_tc_kernel<MODE, 1>, (const void *)conv_tc_kernel<MODE, 2>,
+                          (const void *)conv_tc_kernel<MODE, 4>, (const void *)conv_tc_kernel<MODE, 8>})
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CV_SMEM);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(conv2_tc_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CV2_SMEM);
+    return e;
+}
+
+template <int SPLIT>
+cudaLaunchConfig_t cluster_config(int ctas, cudaStream_t st, cudaLaunchAttribute *attr) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(CV_THREADS);
+    cfg.dynamicSmemBytes = CV_SMEM;
+    cfg.stream = st;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = SPLIT;
+    attr->val.clusterDim.y = 1;
+    attr->val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = SPLIT > 1 ? 1 : 0;
+    return cfg;
+}
+
+template <int SPLIT>
+cudaError_t count_clusters(int nsm, int *n) {
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = cluster_config<SPLIT>(SPLIT * nsm, nullptr, &attr);
+    return cudaOccupancyMaxActiveClusters(n, conv_tc_kernel<CONV_FWD, SPLIT>, &cfg);
+}
+
+// once per device (the last one used is remembered)
+cudaError_t setup() {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     std::lock_guard<std::mutex> lk(g_mu);
-    if (g_attr_device != dev) {
-        if ((e = cudaFuncSetAttribute(conv_tc_kernel<CONV_FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)CV_SMEM)) != cudaSuccess ||
-            (e = cudaFuncSetAttribute(conv_tc_kernel<CONV_DGRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)CV_SMEM)) != cudaSuccess ||
-            (e = cudaFuncSetAttribute(conv_tc_kernel<CONV_WGRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)CV_SMEM)) != cudaSuccess)
-            return e;
-        g_attr_device = dev;
-    }
+    if (g_attr_device == dev) return cudaSuccess;
+    if ((e = cudaDeviceGetAttribute(&g_sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+        (e = setup_mode<CONV_FWD>()) != cudaSuccess || (e = setup_mode<CONV_DGRAD>()) != cudaSuccess ||
+        (e = setup_mode<CONV_WGRAD>()) != cudaSuccess)
+        return e;
+    g_clusters[0] = g_sms;
+    if ((e = count_clusters<2>(g_sms, &g_clusters[1])) != cudaSuccess ||
+        (e = count_clusters<4>(g_sms, &g_clusters[2])) != cudaSuccess ||
+        (e = count_clusters<8>(g_sms, &g_clusters[3])) != cudaSuccess)
+        return e;
+    g_attr_device = dev;
     return cudaSuccess;
 }
 
@@ -66,6 +103,7 @@ ConvArgs make_args(const wici_conv_shape *s, float *out, void *ws) {
     a.pt = (a.p + 7) / 8;
     a.qt = (a.q + 15) / 16;
     a.out = out;
+    a.wide = ((uintptr_t)out & 31u) == 0;
     a.err = (int *)ws;
     return a;
 }
@@ -89,20 +127,62 @@ bool map_dy(CUtensorMap *m, const void *dy, const wici_conv_shape *s, int pbox) 
     return encode_tiled(m, 4, dy, dims, st, box, es);
 }
 
-// a row-major bf16 matrix [rows][cols]: boxes of 64 columns x 256 rows
-bool map_rows(CUtensorMap *m, const void *ptr, uint64_t rows, uint64_t cols) {
+// a row-major bf16 matrix [rows][cols]: boxes of 64 columns x `box_rows` rows
+bool map_rows(CUtensorMap *m, const void *ptr, uint64_t rows, uint64_t cols, int box_rows) {
     const uint64_t dims[2] = {cols, rows};
     const uint64_t st[1] = {cols * 2};
-    const uint32_t box[2] = {64, (uint32_t)CV_BN};
+    const uint32_t box[2] = {64, (uint32_t)box_rows};
     const uint32_t es[2] = {1, 1};
     return encode_tiled(m, 2, ptr, dims, st, box, es);
 }
 
+// How a layer's `tiles` of 128 x 256 outputs with `nkb` reduction blocks (the longest tile's)
+// run: on pairs of CTAs (0), one CTA a tile (1), or 2, 4 or 8 CTAs sharing one.  Modelled
+// SM cycles: waves of tiles x (blocks of a CTA x 512 cycles of MMAs + the pipeline's fill
+// and the epilogue, and the exchange of a split tile).  A single CTA takes about 640
+// cycles a block (its ports serve all of B), a pair 540.
+int pick_ctas(int tiles, int pair_tiles, int nkb) {
+    auto cost = [](int units, int slots, double blocks, double cycles, double fixed) {
+        return (double)((units + slots - 1) / slots) * (blocks * cycles + fixed);
+    };
+    int best = 0;
+    double best_cost = cost(pair_tiles, g_clusters[1], nkb, 540.0, 5000.0);
+    for (int i = 0; i < 4; ++i) {
+        if (g_clusters[i] == 0) continue;
+        const int split = 1 << i;
+        const double c = cost(tiles, g_clusters[i], (nkb + split - 1) / split, 640.0, i == 0 ? 4000.0 : 7000.0);
+        if (c < best_cost) {
+            best = split;
+            best_cost = c;
+        }
+    }
+    return best;
+}
+
+template <int MODE, int SPLIT>
+cudaError_t launch_split(const CUtensorMap &ma, const CUtensorMap &mb, const ConvArgs &a, cudaStream_t st) {
+    cudaLaunchAttribute attr;
+    // one tile per cluster where tiles are shared, otherwise persistent
+    const cudaLaunchConfig_t cfg =
+        cluster_config<SPLIT>(SPLIT > 1 ? a.ntiles * SPLIT : a.ntiles < g_sms ? a.ntiles : g_sms, st, &attr);
+    return cudaLaunchKernelEx(&cfg, conv_tc_kernel<MODE, SPLIT>, ma, mb, a);
+}
+
+// ctas: pick_ctas; mb: boxes of 128 rows for pairs, of 256 otherwise (the same for the filter gradient)
 template <int MODE>
-cudaError_t launch(const CUtensorMap &ma, const CUtensorMap &mb, ConvArgs a, int nsm, cudaStream_t st) {
-    const int grid = a.ntiles < nsm ? a.ntiles : nsm;
-    conv_tc_kernel<MODE><<<grid, CV_THREADS, CV_SMEM, st>>>(ma, mb, a);
-    return cudaGetLastError();
+cudaError_t launch(int ctas, const CUtensorMap &ma, const CUtensorMap &mb, ConvArgs a, int tiles, cudaStream_t st) {
+    a.ntiles = ctas == 0 ? cv_pair_tiles<MODE>(a) : tiles;
+    switch (ctas) {
+        case 0: {
+            const int grid = 2 * (a.ntiles < g_clusters[1] ? a.ntiles : g_clusters[1]);
+            conv2_tc_kernel<MODE><<<grid, CV_THREADS, CV2_SMEM, st>>>(ma, mb, a);
+            return cudaGetLastError();
+        }
+        case 1: return launch_split<MODE, 1>(ma, mb, a, st);
+        case 2: return launch_split<MODE, 2>(ma, mb, a, st);
+        case 4: return launch_split<MODE, 4>(ma, mb, a, st);
+        default: return launch_split<MODE, 8>(ma, mb, a, st);
+    }
 }
 
 }  // namespace
@@ -121,15 +201,16 @@ int wici_conv_forward(void *cuda_stream, const wici_conv_shape *s, const void *x
     if (const char *m = check_shape(s)) return fail(WICI_E_ARG, "conv: %s", m);
     if (!aligned16(x) || !aligned16(w) || !aligned16(y) || !aligned16(workspace) || !workspace)
         return fail(WICI_E_ARG, "conv: null or unaligned buffer");
-    int nsm = 0;
-    cudaError_t e = setup(&nsm);
+    cudaError_t e = setup();
     if (e != cudaSuccess) return fail(WICI_E_CUDA, "conv: %s", cudaGetErrorString(e));
     CUtensorMap ma, mb;
-    if (!map_x_strided(&ma, x, s, 32, 16) || !map_rows(&mb, w, (uint64_t)s->k, (uint64_t)9 * s->c))
+    const ConvArgs a = make_args(s, y, workspace);
+    const int tiles = a.n * a.pt * a.qt * (a.k / CV_BN);
+    const int ctas = pick_ctas(tiles, cv_pair_tiles<CONV_FWD>(a), 9 * (a.c / CV_BK));
+    if (!map_x_strided(&ma, x, s, 32, 16) ||
+        !map_rows(&mb, w, (uint64_t)s->k, (uint64_t)9 * s->c, ctas == 0 ? CV_BN / 2 : CV_BN))
         return fail(WICI_E_CUDA, "conv: cuTensorMapEncodeTiled failed");
-    ConvArgs a = make_args(s, y, workspace);
-    a.ntiles = a.n * a.pt * a.qt * (a.k / CV_BN);
-    if ((e = launch<CONV_FWD>(ma, mb, a, nsm, (cudaStream_t)cuda_stream)) != cudaSuccess)
+    if ((e = launch<CONV_FWD>(ctas, ma, mb, a, tiles, (cudaStream_t)cuda_stream)) != cudaSuccess)
         return fail(WICI_E_CUDA, "conv forward: %s", cudaGetErrorString(e));
     return WICI_OK;
 }
@@ -139,8 +220,7 @@ int wici_conv_backward_data(void *cuda_stream, const wici_conv_shape *s, const v
     if (const char *m = check_shape(s)) return fail(WICI_E_ARG, "conv: %s", m);
     if (!aligned16(dy) || !aligned16(w) || !aligned16(dx) || !aligned16(workspace) || !workspace)
         return fail(WICI_E_ARG, "conv: null or unaligned buffer");
-    int nsm = 0;
-    cudaError_t e = setup(&nsm);
+    cudaError_t e = setup();
     if (e != cudaSuccess) return fail(WICI_E_CUDA, "conv: %s", cudaGetErrorString(e));
     cudaStream_t st = (cudaStream_t)cuda_stream;
     uint16_t *wt = (uint16_t *)((uint8_t *)workspace + kConvErrBytes);
@@ -148,11 +228,13 @@ int wici_conv_backward_data(void *cuda_stream, const wici_conv_shape *s, const v
         (const uint16_t *)w, wt, s->k, s->c);
     if ((e = cudaGetLastError()) != cudaSuccess) return fail(WICI_E_CUDA, "conv transpose: %s", cudaGetErrorString(e));
     CUtensorMap ma, mb;
-    if (!map_dy(&ma, dy, s, 8) || !map_rows(&mb, wt, (uint64_t)9 * s->c, (uint64_t)s->k))
+    const ConvArgs a = make_args(s, dx, workspace);
+    const int tiles = 4 * a.n * a.pt * a.qt * (a.c / CV_BN);
+    const int ctas = pick_ctas(tiles, cv_pair_tiles<CONV_DGRAD>(a), 4 * (a.k / CV_BK));
+    if (!map_dy(&ma, dy, s, 8) ||
+        !map_rows(&mb, wt, (uint64_t)9 * s->c, (uint64_t)s->k, ctas == 0 ? CV_BN / 2 : CV_BN))
         return fail(WICI_E_CUDA, "conv: cuTensorMapEncodeTiled failed");
-    ConvArgs a = make_args(s, dx, workspace);
-    a.ntiles = 4 * a.n * a.pt * a.qt * (a.c / CV_BN);
-    if ((e = launch<CONV_DGRAD>(ma, mb, a, nsm, st)) != cudaSuccess)
+    if ((e = launch<CONV_DGRAD>(ctas, ma, mb, a, tiles, st)) != cudaSuccess)
         return fail(WICI_E_CUDA, "conv data gradient: %s", cudaGetErrorString(e));
     return WICI_OK;
 }
@@ -162,15 +244,15 @@ int wici_conv_backward_filter(void *cuda_stream, const wici_conv_shape *s, const
     if (const char *m = check_shape(s)) return fail(WICI_E_ARG, "conv: %s", m);
     if (!aligned16(x) || !aligned16(dy) || !aligned16(dw) || !aligned16(workspace) || !workspace)
         return fail(WICI_E_ARG, "conv: null or unaligned buffer");
-    int nsm = 0;
-    cudaError_t e = setup(&nsm);
+    cudaError_t e = setup();
     if (e != cudaSuccess) return fail(WICI_E_CUDA, "conv: %s", cudaGetErrorString(e));
     CUtensorMap ma, mb;
     if (!map_dy(&ma, dy, s, 4) || !map_x_strided(&mb, x, s, 32, 8))
         return fail(WICI_E_CUDA, "conv: cuTensorMapEncodeTiled failed");
-    ConvArgs a = make_args(s, dw, workspace);
-    a.ntiles = 9 * (a.k / CV_BM) * (a.c / CV_BN);
-    if ((e = launch<CONV_WGRAD>(ma, mb, a, nsm, (cudaStream_t)cuda_stream)) != cudaSuccess)
+    const ConvArgs a = make_args(s, dw, workspace);
+    const int tiles = 9 * (a.k / CV_BM) * (a.c / CV_BN);
+    const int ctas = pick_ctas(tiles, cv_pair_tiles<CONV_WGRAD>(a), a.n * ((a.p + 3) / 4) * a.qt);
+    if ((e = launch<CONV_WGRAD>(ctas, ma, mb, a, tiles, (cudaStream_t)cuda_stream)) != cudaSuccess)
         return fail(WICI_E_CUDA, "conv filter gradient: %s", cudaGetErrorString(e));
     return WICI_OK;
 }

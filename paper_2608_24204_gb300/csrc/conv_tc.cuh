@@ -20,6 +20,10 @@
 //              (4 output rows x 16 columns).  Both operands are pixel-by-channel
 //              tiles, i.e. MN-major for tcgen05.
 //
+// Few tiles (small layers): with SPLIT = 2, 4 or 8 a cluster of CTAs shares one tile,
+// each over a range of the reduction blocks; the CTAs then exchange column slices of
+// their sums through shared memory, add them in rank order and store their slices.
+// Large layers run on pairs of SMs (conv2_tc.cuh).
 // Persistent, one CTA per SM, three warp roles as in the prefill GEMM: warp 0
 // issues the TMA loads into a 4-stage ring (16 KB A + 32 KB B a stage), warp 1
 // allocates 512 TMEM columns (two 256-column accumulators) and issues
@@ -50,6 +54,7 @@ struct ConvArgs {
     int n, c, h, w, k, p, q;
     int pt, qt;          // output-row tiles (8 rows) and column tiles (16 columns)
     int ntiles;
+    bool wide;           // out is 32-byte aligned
     float *out;          // y [N][P][Q][K], dx [N][H][W][C] or dw [K][3][3][C]
     int *err;
 };
@@ -89,6 +94,20 @@ __device__ __forceinline__ void cv_class(int cls, int &ph, int &pw) {
 __device__ __forceinline__ int cv_ntaps_1d(int ph) { return ph ? 2 : 1; }
 // i-th tap index along one axis of a class: even phase -> r = 1; odd -> r = 0, 2
 __device__ __forceinline__ int cv_tap_1d(int ph, int i) { return ph ? 2 * i : 1; }
+
+// Eight consecutive fp32.  Lanes hold rows far apart, so one 32-byte store per lane writes
+// whole sectors where two 16-byte ones write halves; `wide`: the output is 32-byte
+// aligned (callers promise 16).
+__device__ __forceinline__ void st_global_8(float *p, const float *v, bool wide) {
+    if (!wide) {
+        reinterpret_cast<float4 *>(p)[0] = make_float4(v[0], v[1], v[2], v[3]);
+        reinterpret_cast<float4 *>(p)[1] = make_float4(v[4], v[5], v[6], v[7]);
+        return;
+    }
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+                 "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+                 : "memory");
+}
 
 // tile -> (mode-specific) coordinates; the reduction length in 64-wide blocks
 struct CvTile {
@@ -161,7 +180,20 @@ __device__ __forceinline__ void cv_load(const ConvArgs &a, const CvTile &s, int 
     }
 }
 
+// this thread's output row of tile s (tile row m), its columns from the tile's first;
+// nullptr outside the image
 template <int MODE>
+__device__ __forceinline__ float *cv_row(const ConvArgs &a, const CvTile &s, int m) {
+    if constexpr (MODE == CONV_WGRAD) return a.out + ((size_t)(s.mt * CV_BM + m) * 9 + s.tap) * a.c + s.nt * CV_BN;
+    const int i = s.p0 + m / 16, j = s.q0 + m % 16;
+    if (s.n >= a.n || i >= a.p || j >= a.q) return nullptr;
+    if constexpr (MODE == CONV_FWD)
+        return a.out + (((size_t)s.n * a.p + i) * a.q + j) * a.k + s.nt * CV_BN;
+    else
+        return a.out + (((size_t)s.n * a.h + 2 * i + s.ph) * a.w + 2 * j + s.pw) * a.c + s.nt * CV_BN;
+}
+
+template <int MODE, int SPLIT>
 __global__ void __launch_bounds__(CV_THREADS, 1)
     conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                    const ConvArgs a) {
@@ -172,6 +204,8 @@ __global__ void __launch_bounds__(CV_THREADS, 1)
     __shared__ int s_issued;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    // this CTA's tiles, and its range of a tile's reduction blocks
+    const int rank = (int)blockIdx.x % SPLIT, tile0 = (int)blockIdx.x / SPLIT, tile_step = (int)gridDim.x / SPLIT;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < CV_STAGES; ++s) {
@@ -200,9 +234,10 @@ __global__ void __launch_bounds__(CV_THREADS, 1)
         if (lane == 0) {  // ------------------------------------------- TMA producer
             int it = 0;
             bool ok = true;
-            for (int t = blockIdx.x; t < a.ntiles && ok; t += gridDim.x) {
+            for (int t = tile0; t < a.ntiles && ok; t += tile_step) {
                 const CvTile s = cv_tile<MODE>(a, t);
-                for (int kb = 0; kb < s.nkb; ++kb, ++it) {
+                const int kb1 = (rank + 1) * s.nkb / SPLIT;
+                for (int kb = rank * s.nkb / SPLIT; kb < kb1; ++kb, ++it) {
                     const int st = it % CV_STAGES;
                     if (it >= CV_STAGES &&
                         !(ok = mbar_wait(smem_u32(&empty_bar[st]), ((it / CV_STAGES) + 1) & 1, a.err, SITE_CV_EMPTY)))
@@ -220,14 +255,15 @@ __global__ void __launch_bounds__(CV_THREADS, 1)
             constexpr uint32_t idesc = cv_idesc(MN);
             bool ok = true;
             int it = 0, tt = 0;
-            for (int t = blockIdx.x; t < a.ntiles && ok; t += gridDim.x, ++tt) {
+            for (int t = tile0; t < a.ntiles && ok; t += tile_step, ++tt) {
                 const CvTile s = cv_tile<MODE>(a, t);
                 const int b = tt & 1;
                 if (tt >= 2 && !(ok = mbar_wait(smem_u32(&acc_free[b]), ((tt / 2) + 1) & 1, a.err, SITE_CV_FREE)))
                     break;
                 tc_fence_after();
                 const uint32_t acc = tmem + (uint32_t)(b * CV_BN);
-                for (int kb = 0; kb < s.nkb; ++kb, ++it) {
+                const int kb0 = rank * s.nkb / SPLIT, kb1 = (rank + 1) * s.nkb / SPLIT;
+                for (int kb = kb0; kb < kb1; ++kb, ++it) {
                     const int st = it % CV_STAGES;
                     ok = mbar_wait(smem_u32(&full_bar[st]), (it / CV_STAGES) & 1, a.err, SITE_CV_FULL);
                     if (!ok) break;
@@ -243,7 +279,7 @@ __global__ void __launch_bounds__(CV_THREADS, 1)
                             ad = tc_desc_sw128(sa + 32u * k);
                             bd = tc_desc_sw128(sb + 32u * k);
                         }
-                        tc_mma(acc, ad, bd, idesc, (kb | k) != 0);
+                        tc_mma(acc, ad, bd, idesc, kb != kb0 || k != 0);
                     }
                     tc_commit(smem_u32(&empty_bar[st]));
                 }
@@ -256,35 +292,73 @@ __global__ void __launch_bounds__(CV_THREADS, 1)
         const int m = qd * 32 + lane;                   // tile row = TMEM lane
         const uint32_t lane_base = (uint32_t)(qd * 32) << 16;
         int tt = 0;
-        for (int t = blockIdx.x; t < a.ntiles; t += gridDim.x, ++tt) {
+        bool ok = true;
+        for (int t = tile0; t < a.ntiles && ok; t += tile_step, ++tt) {
             const CvTile s = cv_tile<MODE>(a, t);
             const int b = tt & 1;
-            if (!mbar_wait(smem_u32(&acc_full[b]), (tt / 2) & 1, a.err, SITE_CV_ACCUM)) break;
+            ok = mbar_wait(smem_u32(&acc_full[b]), (tt / 2) & 1, a.err, SITE_CV_ACCUM);
             tc_fence_after();
-            float *row = nullptr;     // this thread's output row, columns from the tile's first
-            if constexpr (MODE == CONV_FWD) {
-                const int p = s.p0 + m / 16, q = s.q0 + m % 16;
-                if (p < a.p && q < a.q) row = a.out + (((size_t)s.n * a.p + p) * a.q + q) * a.k + s.nt * CV_BN;
-            } else if constexpr (MODE == CONV_DGRAD) {
-                const int i = s.p0 + m / 16, j = s.q0 + m % 16;
-                if (i < a.p && j < a.q)
-                    row = a.out + (((size_t)s.n * a.h + 2 * i + s.ph) * a.w + 2 * j + s.pw) * a.c + s.nt * CV_BN;
+            float *row = cv_row<MODE>(a, s, m);
+            const uint32_t ta = tmem + lane_base + (uint32_t)(b * CV_BN + half * (CV_BN / 2));
+            if constexpr (SPLIT == 1) {
+                if (!ok) break;
+#pragma unroll
+                for (int c0 = 0; c0 < CV_BN / 2; c0 += 32) {
+                    float v[32];
+                    tc_ld32(ta + (uint32_t)c0, v);
+                    if (row) {
+#pragma unroll
+                        for (int i = 0; i < 32; i += 8) st_global_8(row + half * (CV_BN / 2) + c0 + i, v + i, a.wide);
+                    }
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&acc_free[b]));
             } else {
-                row = a.out + ((size_t)(s.mt * CV_BM + m) * 9 + s.tap) * a.c + s.nt * CV_BN;
-            }
+                // one tile per CTA: every CTA of the cluster has finished with its ring, so the
+                // sums' column slices cross through it: [source rank][row][SL + 4]
+                constexpr int SL = CV_BN / SPLIT, PITCH = SL + 4;
+                constexpr uint32_t SRC = CV_BM * PITCH * 4;
+                static_assert(SPLIT * SRC <= CV_STAGES * CV_STAGE_BYTES, "slices fit the ring");
+                const bool some = (rank + 1) * s.nkb / SPLIT > rank * s.nkb / SPLIT;   // else nothing was accumulated
+                cluster_sync_all();
 #pragma unroll
-            for (int c0 = 0; c0 < CV_BN / 2; c0 += 32) {
-                float v[32];
-                tc_ld32(tmem + lane_base + (uint32_t)(b * CV_BN + half * (CV_BN / 2) + c0), v);
-                if (row) {
-                    float4 *dst = reinterpret_cast<float4 *>(row + half * (CV_BN / 2) + c0);
+                for (int c0 = 0; c0 < CV_BN / 2; c0 += 32) {
+                    float v[32];
+                    tc_ld32(ta + (uint32_t)c0, v);
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) dst[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+                    for (int i = 0; i < 32; i += 4) {
+                        const int col = half * (CV_BN / 2) + c0 + i;
+                        st_cluster_v4(base + (uint32_t)rank * SRC + (uint32_t)(m * PITCH + col % SL) * 4, col / SL,
+                                      some ? v[i] : 0.f, some ? v[i + 1] : 0.f, some ? v[i + 2] : 0.f,
+                                      some ? v[i + 3] : 0.f);
+                    }
+                }
+                cluster_sync_all();
+                constexpr int NC = SL / 2;   // columns of the slice per warp of a pair
+                const uint8_t *src = smem_raw + (base - smem_u32(smem_raw)) + (size_t)(m * PITCH + half * NC) * 4;
+                if (ok && row) {
+#pragma unroll
+                    for (int c = 0; c < NC; c += 8) {
+                        float v[8] = {};
+#pragma unroll
+                        for (int r = 0; r < SPLIT; ++r) {
+                            const float4 x = *reinterpret_cast<const float4 *>(src + r * SRC + c * 4);
+                            const float4 y = *reinterpret_cast<const float4 *>(src + r * SRC + c * 4 + 16);
+                            v[0] += x.x; v[1] += x.y; v[2] += x.z; v[3] += x.w;
+                            v[4] += y.x; v[5] += y.y; v[6] += y.z; v[7] += y.w;
+                        }
+                        st_global_8(row + rank * SL + half * NC + c, v, a.wide);
+                    }
                 }
             }
-            tc_fence_before();
+        }
+    }
+    if constexpr (SPLIT > 1) {
+        if (warp < 2) {   // the epilogue warps' two cluster barriers count every thread
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&acc_free[b]));
+            cluster_sync_all();
+            cluster_sync_all();
         }
     }
     tc_fence_before();
