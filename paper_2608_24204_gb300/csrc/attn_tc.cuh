@@ -216,6 +216,8 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_tmem;
+    griddep_launch_dependents();
+    griddep_wait();
     const uint32_t tm_q = tmem + TM::Q, tm_sp = tmem + TM::SP, tm_o = tmem + TM::O;
 
     if (warp == 0) {

@@ -142,6 +142,36 @@ __device__ __forceinline__ void griddep_launch_dependents() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// Host: launch on `st`, in clusters of `cluster` CTAs, optionally before the stream's
+// previous kernel has finished (`pdl`: the kernel runs griddep_wait before it touches
+// what earlier kernels wrote or read).
+template <typename Kern, typename... Args>
+cudaError_t launch_kernel(Kern kern, dim3 grid, int threads, size_t smem, cudaStream_t st, int cluster, bool pdl,
+                          const Args &...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    unsigned n = 0;
+    if (cluster > 1) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = cluster;
+        attr[n].val.clusterDim.y = 1;
+        attr[n].val.clusterDim.z = 1;
+        ++n;
+    }
+    if (pdl) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n].val.programmaticStreamSerializationAllowed = 1;
+        ++n;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = n;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 // -------------------------------------------------------------- misc ----
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll

@@ -54,25 +54,18 @@ cudaError_t setup_mode() {
 }
 
 template <int SPLIT>
-cudaLaunchConfig_t cluster_config(int ctas, cudaStream_t st, cudaLaunchAttribute *attr) {
+cudaError_t count_clusters(int nsm, int *n) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(ctas);
+    cfg.gridDim = dim3(SPLIT * nsm);
     cfg.blockDim = dim3(CV_THREADS);
     cfg.dynamicSmemBytes = CV_SMEM;
-    cfg.stream = st;
-    attr->id = cudaLaunchAttributeClusterDimension;
-    attr->val.clusterDim.x = SPLIT;
-    attr->val.clusterDim.y = 1;
-    attr->val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = SPLIT > 1 ? 1 : 0;
-    return cfg;
-}
-
-template <int SPLIT>
-cudaError_t count_clusters(int nsm, int *n) {
     cudaLaunchAttribute attr;
-    const cudaLaunchConfig_t cfg = cluster_config<SPLIT>(SPLIT * nsm, nullptr, &attr);
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = SPLIT;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
     return cudaOccupancyMaxActiveClusters(n, conv_tc_kernel<CONV_FWD, SPLIT>, &cfg);
 }
 
@@ -161,11 +154,9 @@ int pick_ctas(int tiles, int pair_tiles, int nkb) {
 
 template <int MODE, int SPLIT>
 cudaError_t launch_split(const CUtensorMap &ma, const CUtensorMap &mb, const ConvArgs &a, cudaStream_t st) {
-    cudaLaunchAttribute attr;
     // one tile per cluster where tiles are shared, otherwise persistent
-    const cudaLaunchConfig_t cfg =
-        cluster_config<SPLIT>(SPLIT > 1 ? a.ntiles * SPLIT : a.ntiles < g_sms ? a.ntiles : g_sms, st, &attr);
-    return cudaLaunchKernelEx(&cfg, conv_tc_kernel<MODE, SPLIT>, ma, mb, a);
+    const int grid = SPLIT > 1 ? a.ntiles * SPLIT : a.ntiles < g_sms ? a.ntiles : g_sms;
+    return launch_kernel(conv_tc_kernel<MODE, SPLIT>, dim3(grid), CV_THREADS, CV_SMEM, st, SPLIT, true, ma, mb, a);
 }
 
 // ctas: pick_ctas; mb: boxes of 128 rows for pairs, of 256 otherwise (the same for the filter gradient)
@@ -175,8 +166,8 @@ cudaError_t launch(int ctas, const CUtensorMap &ma, const CUtensorMap &mb, ConvA
     switch (ctas) {
         case 0: {
             const int grid = 2 * (a.ntiles < g_clusters[1] ? a.ntiles : g_clusters[1]);
-            conv2_tc_kernel<MODE><<<grid, CV_THREADS, CV2_SMEM, st>>>(ma, mb, a);
-            return cudaGetLastError();
+            // __cluster_dims__ gives the pairs
+            return launch_kernel(conv2_tc_kernel<MODE>, dim3(grid), CV_THREADS, CV2_SMEM, st, 1, true, ma, mb, a);
         }
         case 1: return launch_split<MODE, 1>(ma, mb, a, st);
         case 2: return launch_split<MODE, 2>(ma, mb, a, st);
@@ -224,9 +215,9 @@ int wici_conv_backward_data(void *cuda_stream, const wici_conv_shape *s, const v
     if (e != cudaSuccess) return fail(WICI_E_CUDA, "conv: %s", cudaGetErrorString(e));
     cudaStream_t st = (cudaStream_t)cuda_stream;
     uint16_t *wt = (uint16_t *)((uint8_t *)workspace + kConvErrBytes);
-    conv_transpose_filter_kernel<<<dim3((s->c + 31) / 32, (s->k + 31) / 32, 9), dim3(32, 8), 0, st>>>(
-        (const uint16_t *)w, wt, s->k, s->c);
-    if ((e = cudaGetLastError()) != cudaSuccess) return fail(WICI_E_CUDA, "conv transpose: %s", cudaGetErrorString(e));
+    if ((e = launch_kernel(conv_transpose_filter_kernel, dim3((s->c + 31) / 32, (s->k + 31) / 32, 9), 256, 0, st, 1, true,
+                           (const uint16_t *)w, wt, s->k, s->c)) != cudaSuccess)
+        return fail(WICI_E_CUDA, "conv transpose: %s", cudaGetErrorString(e));
     CUtensorMap ma, mb;
     const ConvArgs a = make_args(s, dx, workspace);
     const int tiles = 4 * a.n * a.pt * a.qt * (a.c / CV_BN);

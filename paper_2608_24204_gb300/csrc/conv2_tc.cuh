@@ -135,6 +135,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CV_THREADS, 1)
     cluster_sync_all();   // both CTAs' barriers and tensor memory are ready
     tc_fence_after();
     const uint32_t tmem = s_tmem;
+    griddep_launch_dependents();
+    griddep_wait();
 
     if (warp == 0) {
         if (lane == 0) {  // ------------------------------------------- TMA producer

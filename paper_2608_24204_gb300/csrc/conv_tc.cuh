@@ -229,6 +229,8 @@ __global__ void __launch_bounds__(CV_THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_tmem;
+    griddep_launch_dependents();
+    griddep_wait();
 
     if (warp == 0) {
         if (lane == 0) {  // ------------------------------------------- TMA producer
@@ -374,18 +376,20 @@ __global__ void __launch_bounds__(CV_THREADS, 1)
     }
 }
 
-// w [K][9][C] -> w^T [9][C][K] (the data gradient's K-major B operand), 32 x 32 tiles
+// w [K][9][C] -> w^T [9][C][K] (the data gradient's K-major B operand), 32 x 32 tiles, 8 warps
 __global__ void conv_transpose_filter_kernel(const uint16_t *w, uint16_t *wt, int K, int C) {
     __shared__ uint16_t tile[32][33];
-    const int tap = blockIdx.z, k0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int k = k0 + i, c = c0 + threadIdx.x;
-        tile[i][threadIdx.x] = (k < K && c < C) ? w[((size_t)k * 9 + tap) * C + c] : 0;
+    griddep_launch_dependents();
+    griddep_wait();   // an earlier data gradient may still read wt
+    const int lane = threadIdx.x & 31, tap = blockIdx.z, k0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
+    for (int i = threadIdx.x >> 5; i < 32; i += 8) {
+        const int k = k0 + i, c = c0 + lane;
+        tile[i][lane] = (k < K && c < C) ? w[((size_t)k * 9 + tap) * C + c] : 0;
     }
     __syncthreads();
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int c = c0 + i, k = k0 + threadIdx.x;
-        if (c < C && k < K) wt[((size_t)tap * C + c) * K + k] = tile[threadIdx.x][i];
+    for (int i = threadIdx.x >> 5; i < 32; i += 8) {
+        const int c = c0 + i, k = k0 + lane;
+        if (c < C && k < K) wt[((size_t)tap * C + c) * K + k] = tile[lane][i];
     }
 }
 

@@ -117,11 +117,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
     cluster_sync_all();   // both CTAs' barriers and tensor memory are ready
     tc_fence_after();
     const uint32_t tmem = s_tmem;
+    griddep_launch_dependents();
+    if (warp != 0) griddep_wait();   // warp 0 waits behind its first weight copies
 
     if (warp == 0) {
         if (lane == 0) {  // ------------------------------------------- TMA producer
             int it = 0;
             bool ok = true;
+            // as in gemm_tc_kernel: the first bf16 weight copies precede the wait
+            const int early = WT == 1 && tile0 < ntiles ? min(S, nkk) : 0;
+            for (int s = 0; s < early; ++s) {
+                const uint32_t fb = smem_u32(&full_bar[s]);
+                if (rank == 0) mbar_arrive_expect_tx(fb, 2u * (AT * TC_A_BYTES + G::B_BYTES));
+                tma_load_2d_pair(base + (uint32_t)s * G::STAGE_BYTES + AT * TC_A_BYTES, &maps.w[0], s * TC_BK,
+                                 (tile0 / ntm) * BN + rank * (BN / 2), fb);
+            }
+            griddep_wait();
             for (int tile = tile0; tile < ntiles && ok; tile += tile_step) {
                 const int m0 = (tile % ntm) * 2 * TC_BM + rank * TC_BM, n0 = (tile / ntm) * BN + rank * (BN / 2);
                 for (int kk = 0; kk < nkk; ++kk, ++it) {
@@ -133,13 +144,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
                     const uint32_t fb = smem_u32(&full_bar[s]);
                     const int na = AT - j;   // term j meets the activation terms i < AT - j only
                     if (rank == 0) {
-                        mbar_arrive_expect_tx(fb, 2u * ((uint32_t)na * TC_A_BYTES + G::B_BYTES));
+                        if (it >= early) mbar_arrive_expect_tx(fb, 2u * ((uint32_t)na * TC_A_BYTES + G::B_BYTES));
                         s_issued = it + 1;
                     }
 #pragma unroll
                     for (int t = 0; t < AT; ++t)
                         if (t < na) tma_load_2d_pair(st + t * TC_A_BYTES, &maps.a[t], kb * TC_BK, m0, fb);
-                    tma_load_2d_pair(st + AT * TC_A_BYTES, &maps.w[j], kb * TC_BK, n0, fb);
+                    if (it >= early) tma_load_2d_pair(st + AT * TC_A_BYTES, &maps.w[j], kb * TC_BK, n0, fb);
                 }
             }
         }

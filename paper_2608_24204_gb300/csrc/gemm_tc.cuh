@@ -221,14 +221,26 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_tmem;
+    griddep_launch_dependents();
+    if (warp != 0) griddep_wait();   // warp 0 waits behind its first weight copies
 
     if (warp == 0) {
         if (lane == 0) {  // ------------------------------------------- TMA producer
             int it = 0;   // k-blocks issued over all tiles
             bool ok = true;
+            const uint32_t a_bytes = (uint32_t)maps.a_rows * (TC_BK * 2);
+            // a bf16 weight does not depend on the kernels before this one: its first k-blocks
+            // are on their way while those finish (8-bit: dequantised by the kernel before)
+            const int early = WT == 1 && tile0 < ntiles ? min(S, kk_end - kk_begin) : 0;
+            for (int s = 0; s < early; ++s) {
+                const uint32_t fb = smem_u32(&full_bar[s]);
+                mbar_arrive_expect_tx(fb, AT * a_bytes + G::B_BYTES);
+                tma_load_2d(base + (uint32_t)s * G::STAGE_BYTES + AT * TC_A_BYTES, &maps.w[0], (kk_begin + s) * TC_BK,
+                            (tile0 / ntm) * BN, fb);
+            }
+            griddep_wait();
             for (int tile = tile0; tile < ntiles && ok; tile += tile_step) {
                 const int m0 = (tile % ntm) * TC_BM, n0 = (tile / ntm) * BN;
-                const uint32_t a_bytes = (uint32_t)maps.a_rows * (TC_BK * 2);
                 for (int kk = kk_begin; kk < kk_end; ++kk, ++it) {
                     const int s = it % S;
                     if (it >= S && !(ok = mbar_wait(smem_u32(&empty_bar[s]), ((it / S) + 1) & 1, err, SITE_TC_EMPTY)))
@@ -238,11 +250,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                     const uint32_t fb = smem_u32(&full_bar[s]);
                     // term j meets the activation terms i <= 2 - j only
                     const int na = AT - j;
-                    mbar_arrive_expect_tx(fb, (uint32_t)na * a_bytes + G::B_BYTES);
+                    if (it >= early) mbar_arrive_expect_tx(fb, (uint32_t)na * a_bytes + G::B_BYTES);
 #pragma unroll
                     for (int t = 0; t < AT; ++t)
                         if (t < na) tma_load_2d(st + t * TC_A_BYTES, &maps.a[t], kb * TC_BK, m0, fb);
-                    tma_load_2d(st + AT * TC_A_BYTES, &maps.w[j], kb * TC_BK, n0, fb);
+                    if (it >= early) tma_load_2d(st + AT * TC_A_BYTES, &maps.w[j], kb * TC_BK, n0, fb);
                     s_issued = it + 1;
                 }
             }

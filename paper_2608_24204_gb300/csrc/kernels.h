@@ -105,14 +105,13 @@ bool decode_is_persistent(const Plan &p);
 cudaError_t enqueue_decode_step(const Plan &p, const Bufs &b, const CUtensorMap &map_kv, cudaStream_t st, bool pdl,
                                 LaunchHook *hook);
 
-// Final RMSNorm + LM head + argmax of the row in b.x; the last CTA writes
+// Final RMSNorm + LM head + argmax of the row x [H]; the last CTA writes
 // ctrl[CTRL_TOKEN], hist[pos + pos_add] and advances ctrl[CTRL_POS] by pos_add.
-cudaError_t enqueue_lm_head(const Plan &p, const Bufs &b, cudaStream_t st, bool pdl, int pos_add,
+cudaError_t enqueue_lm_head(const Plan &p, const Bufs &b, const float *x, cudaStream_t st, bool pdl, int pos_add,
                             LaunchHook *hook);
 
 // Prefill of the chunk b.tok[0..T) at positions P..P+T-1 through every layer.
-// With lm_pos_add > 0 it then copies the chunk's last row to b.x and runs the
-// LM head, which advances ctrl[CTRL_POS] by lm_pos_add.
+// With lm_pos_add > 0 it then runs the LM head on the chunk's last row, which advances ctrl[CTRL_POS] by lm_pos_add.
 cudaError_t enqueue_prefill_chunk(const Plan &p, const Bufs &b, const PrefillMaps &maps,
                                   cudaStream_t st, int P, int T, int lm_pos_add, LaunchHook *hook);
 

@@ -2208,9 +2208,9 @@ static void set_next(const Plan &p, const Bufs &b, GemvIn &g, int layer, int id)
     }
 }
 
-cudaError_t enqueue_lm_head(const Plan &p, const Bufs &b, cudaStream_t st, bool pdl, int pos_add,
+cudaError_t enqueue_lm_head(const Plan &p, const Bufs &b, const float *x, cudaStream_t st, bool pdl, int pos_add,
                             LaunchHook *hook) {
-    GemvIn g = gemv_in(p, b, b.W + p.w_lm, p.H, p.V, 1, b.x, b.W + p.w_final_norm);
+    GemvIn g = gemv_in(p, b, b.W + p.w_lm, p.H, p.V, 1, x, b.W + p.w_final_norm);
     set_next(p, b, g, p.L - 1, G_LM);   // a decode step (layer 0) follows
     EpiArgmax e = {};
     e.logits = b.logits;
@@ -2403,7 +2403,7 @@ cudaError_t enqueue_decode_step(const Plan &p, const Bufs &b, const CUtensorMap 
             return e;
     }
     // A9: final norm + LM head + greedy argmax; advances the position by one
-    return enqueue_lm_head(p, b, st, pdl, 1, hook);
+    return enqueue_lm_head(p, b, b.x, st, pdl, 1, hook);
 }
 
 cudaError_t enqueue_bounded_wait_probe(int *err, int64_t limit_ns, cudaStream_t st) {

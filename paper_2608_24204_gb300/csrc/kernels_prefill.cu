@@ -83,6 +83,8 @@ struct Terms {   // kTerms pointers passed by value to kernels
 
 // ----------------------------------------------------------- embed / norm ----
 __global__ void embed_rows_kernel(const uint16_t *E, const int *tok, float *X, int H) {
+    griddep_launch_dependents();
+    griddep_wait();
     const int t = blockIdx.x;
     const uint16_t *row = E + (size_t)tok[t] * H;
     for (int i = threadIdx.x; i < H; i += blockDim.x) X[(size_t)t * H + i] = bf16_to_f32(row[i]);
@@ -95,6 +97,8 @@ __global__ void embed_rows_kernel(const uint16_t *E, const int *tok, float *X, i
 __global__ void rmsnorm_rows_kernel(const float *X, const uint16_t *g, const Terms A, int H, float eps,
                                     int nterms) {
     __shared__ float s_part[32];
+    griddep_launch_dependents();
+    griddep_wait();
     const int t = blockIdx.x;
     const float4 *x = reinterpret_cast<const float4 *>(X + (size_t)t * H);
     const int nc = H >> 3;
@@ -349,6 +353,8 @@ __global__ void qk_norm_rope_kernel(const float *raw, const uint16_t *qn, const 
                                     Terms Q, uint16_t *kv, const int *pages, size_t page_elems, int P, int nq,
                                     int nkv, float eps) {
     constexpr int EPL = D / 32, HALF = D / 2;
+    griddep_launch_dependents();
+    griddep_wait();
     const int t = blockIdx.x, lane = threadIdx.x & 31;
     const int hd = blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (hd >= nq + nkv) return;
@@ -392,6 +398,8 @@ __global__ void qk_norm_rope_kernel(const float *raw, const uint16_t *qn, const 
 // significant bits), and so is its split into three terms.  8 elements per
 // thread: one 8-byte code load, one scale, one 16-byte store per term.
 __global__ void q8_dequant_terms_kernel(const uint8_t *src, int rows, int K, const Terms out, int nterms) {
+    griddep_launch_dependents();
+    griddep_wait();   // the GEMM before still reads the terms of its matrix
     const int per_row = K / 8;
     const size_t rb = (size_t)K + (size_t)K / 16;
     const long long n = (long long)rows * per_row;
@@ -425,10 +433,11 @@ static cudaError_t dequant_terms(const Plan &p, const Bufs &b, const uint16_t *W
     const long long n = (long long)rows * (K / 8);
     const int grid = (int)((n + 255) / 256 < 8 * p.num_sms ? (n + 255) / 256 : 8 * p.num_sms);
     if (hook) hook->before("prefill_q8_dequant");
-    q8_dequant_terms_kernel<<<grid, 256, 0, st>>>(reinterpret_cast<const uint8_t *>(W), rows, K,
-                                                 Terms{{b.Wt[0], b.Wt[1], b.Wt[2]}}, nterms);
+    const cudaError_t e =
+        launch_kernel(q8_dequant_terms_kernel, dim3(grid), 256, 0, st, 1, true, reinterpret_cast<const uint8_t *>(W), rows,
+                      K, Terms{{b.Wt[0], b.Wt[1], b.Wt[2]}}, nterms);
     if (hook) hook->after("prefill_q8_dequant");
-    return cudaGetLastError();
+    return e;
 }
 
 // --------------------------------------------------------------- RoPE table --
@@ -622,10 +631,8 @@ cudaError_t launch_attn_tc(const Plan &p, const Bufs &b, const PrefillMaps &mp, 
     a.scale_log2 = 1.4426950408889634f / sqrtf((float)p.d);
     dim3 grid(((T + a.tpt - 1) / a.tpt) * p.nkv);
     if (p.d == 128)
-        attn_tc_kernel<128><<<grid, AT_THREADS, AttnSmem<128>::TOTAL + 1024, st>>>(mp.kv, a);
-    else
-        attn_tc_kernel<64><<<grid, AT_THREADS, AttnSmem<64>::TOTAL + 1024, st>>>(mp.kv, a);
-    return cudaGetLastError();
+        return launch_kernel(attn_tc_kernel<128>, grid, AT_THREADS, AttnSmem<128>::TOTAL + 1024, st, 1, true, mp.kv, a);
+    return launch_kernel(attn_tc_kernel<64>, grid, AT_THREADS, AttnSmem<64>::TOTAL + 1024, st, 1, true, mp.kv, a);
 }
 
 // the weight operand of one GEMM: one exact bf16 matrix, or three terms
@@ -638,21 +645,14 @@ template <int BN, int SPLIT, class Epi>
 static cudaError_t launch_gemm(const Plan &p, const GemmMaps &maps, int terms, int T, int N, int K, int *err,
                                const Epi &epi, cudaStream_t st) {
     const int tiles = ((T + TC_BM - 1) / TC_BM) * ((N + BN - 1) / BN);
-    cudaLaunchConfig_t cfg = {};
     // persistent, at most one CTA per SM; a split tile's CTAs are one cluster
-    cfg.gridDim = dim3(SPLIT > 1 ? tiles * SPLIT : tiles < p.num_sms ? tiles : p.num_sms);
-    cfg.blockDim = dim3(TC_THREADS);
-    cfg.dynamicSmemBytes = TcTile<BN, Epi::kATerms>::SMEM;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = SPLIT;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = SPLIT > 1 ? 1 : 0;
-    if (terms == 1) return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<BN, SPLIT, 1, Epi>, maps, T, N, K, err, epi);
-    return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<BN, SPLIT, kTerms, Epi>, maps, T, N, K, err, epi);
+    const dim3 grid(SPLIT > 1 ? tiles * SPLIT : tiles < p.num_sms ? tiles : p.num_sms);
+    constexpr size_t smem = TcTile<BN, Epi::kATerms>::SMEM;
+    if (terms == 1)
+        return launch_kernel(gemm_tc_kernel<BN, SPLIT, 1, Epi>, grid, TC_THREADS, smem, st, SPLIT, true, maps, T, N, K, err,
+                             epi);
+    return launch_kernel(gemm_tc_kernel<BN, SPLIT, kTerms, Epi>, grid, TC_THREADS, smem, st, SPLIT, true, maps, T, N, K,
+                         err, epi);
 }
 
 template <int BN, class Epi>
@@ -661,11 +661,12 @@ static cudaError_t launch_gemm_pair(int pairs, const GemmMaps &maps, int terms, 
     const int tiles = ((T + 2 * TC_BM - 1) / (2 * TC_BM)) * ((N + BN - 1) / BN);
     const int grid = 2 * (tiles < pairs ? tiles : pairs);
     constexpr size_t smem = TcPairTile<BN, Epi::kATerms>::SMEM;
+    // __cluster_dims__ gives the pairs
     if (terms == 1)
-        gemm2_tc_kernel<BN, 1, Epi><<<grid, TC_THREADS, smem, st>>>(maps, T, N, K, err, epi);
-    else
-        gemm2_tc_kernel<BN, kTerms, Epi><<<grid, TC_THREADS, smem, st>>>(maps, T, N, K, err, epi);
-    return cudaGetLastError();
+        return launch_kernel(gemm2_tc_kernel<BN, 1, Epi>, dim3(grid), TC_THREADS, smem, st, 1, true, maps, T, N, K, err,
+                             epi);
+    return launch_kernel(gemm2_tc_kernel<BN, kTerms, Epi>, dim3(grid), TC_THREADS, smem, st, 1, true, maps, T, N, K, err,
+                         epi);
 }
 
 // a: the activation's maps with boxes of 32, 64, 96 and 128 rows
@@ -722,14 +723,17 @@ cudaError_t enqueue_prefill_chunk(const Plan &p, const Bufs &b, const PrefillMap
                                   int T, int lm_pos_add, LaunchHook *hook) {
     cudaError_t e;
     int *err = b.ctrl + CTRL_ERR;
-    embed_rows_kernel<<<T, 256, 0, st>>>(b.W + p.w_embed, b.tok, b.X, p.H);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_kernel(embed_rows_kernel, dim3(T), 256, 0, st, 1, true, b.W + p.w_embed, b.tok, b.X, p.H)) !=
+        cudaSuccess)
+        return e;
     for (int l = 0; l < p.L; ++l) {
         const LayerOffsets &lo = p.layer[l];
         uint16_t *kvl = b.KV + (size_t)l * p.kv_layer_elems;
         // A3 + A4: RMSNorm, QKV (+bias), RoPE, paged KV append
         const Terms A = {{b.A[0], b.A[1], b.A[2]}};
-        rmsnorm_rows_kernel<<<T, 256, 0, st>>>(b.X, b.W + lo.attn_norm, A, p.H, p.cfg.rms_eps, PEpiQKV::kATerms);
+        if ((e = launch_kernel(rmsnorm_rows_kernel, dim3(T), 256, 0, st, 1, true, b.X, b.W + lo.attn_norm, A, p.H,
+                               p.cfg.rms_eps, PEpiQKV::kATerms)) != cudaSuccess)
+            return e;
         PEpiQKV eq = {{{b.Q[0], b.Q[1], b.Q[2]}}, kvl, b.pages, b.rope, p.cfg.qkv_bias ? b.W + lo.bqkv : nullptr, P, p.qdim,
                       p.kvdim, p.d, p.nkv, p.kv_page_elems, p.qk_norm ? b.QKraw : nullptr};
         WOperand w;
@@ -743,14 +747,11 @@ cudaError_t enqueue_prefill_chunk(const Plan &p, const Bufs &b, const PrefillMap
             const Terms Qt = {{b.Q[0], b.Q[1], b.Q[2]}};
             const dim3 grid(T, (p.nq + p.nkv + 7) / 8);
             if (hook) hook->before("prefill_qk_norm_rope");
-            if (p.d == 128)
-                qk_norm_rope_kernel<128><<<grid, 256, 0, st>>>(b.QKraw, b.W + lo.qn, b.W + lo.kn, b.rope, Qt, kvl,
-                                                               b.pages, p.kv_page_elems, P, p.nq, p.nkv, p.cfg.rms_eps);
-            else
-                qk_norm_rope_kernel<64><<<grid, 256, 0, st>>>(b.QKraw, b.W + lo.qn, b.W + lo.kn, b.rope, Qt, kvl,
-                                                              b.pages, p.kv_page_elems, P, p.nq, p.nkv, p.cfg.rms_eps);
+            e = launch_kernel(p.d == 128 ? qk_norm_rope_kernel<128> : qk_norm_rope_kernel<64>, grid, 256, 0, st, 1, true,
+                              b.QKraw, b.W + lo.qn, b.W + lo.kn, b.rope, Qt, kvl, b.pages, p.kv_page_elems, P, p.nq,
+                              p.nkv, p.cfg.rms_eps);
             if (hook) hook->after("prefill_qk_norm_rope");
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            if (e != cudaSuccess) return e;
         }
         // A5: causal attention over the cache (earlier chunks + this one), tensor cores
         if (hook) hook->before("prefill_attention");
@@ -765,7 +766,9 @@ cudaError_t enqueue_prefill_chunk(const Plan &p, const Bufs &b, const PrefillMap
                       "prefill_o_proj")) != cudaSuccess)
             return e;
         // A7: RMSNorm + gate/up + SwiGLU
-        rmsnorm_rows_kernel<<<T, 256, 0, st>>>(b.X, b.W + lo.ffn_norm, A, p.H, p.cfg.rms_eps, PEpiSwiGLU::kATerms);
+        if ((e = launch_kernel(rmsnorm_rows_kernel, dim3(T), 256, 0, st, 1, true, b.X, b.W + lo.ffn_norm, A, p.H,
+                               p.cfg.rms_eps, PEpiSwiGLU::kATerms)) != cudaSuccess)
+            return e;
         const Terms M = {{b.M[0], b.M[1], b.M[2]}};
         if ((e = weight_operand<PEpiSwiGLU>(p, b, p.q8 ? mp.wt_gu[0] : mp.wgu[l], mp.wt_gu, b.W + lo.wgu, 2 * p.F, p.H, st,
                                 hook, &w)) != cudaSuccess)
@@ -783,10 +786,7 @@ cudaError_t enqueue_prefill_chunk(const Plan &p, const Bufs &b, const PrefillMap
     }
     if (lm_pos_add > 0) {
         // A9 on the chunk's last row only
-        if ((e = cudaMemcpyAsync(b.x, b.X + (size_t)(T - 1) * p.H, (size_t)p.H * sizeof(float),
-                                 cudaMemcpyDeviceToDevice, st)) != cudaSuccess)
-            return e;
-        return enqueue_lm_head(p, b, st, false, lm_pos_add, hook);
+        return enqueue_lm_head(p, b, b.X + (size_t)(T - 1) * p.H, st, true, lm_pos_add, hook);
     }
     return cudaSuccess;
 }
