@@ -63,7 +63,8 @@ def peaks():
                 "source": "fallback"}
 
 
-KERNEL_SOURCES = ["paper_2608_24204_gb300/csrc/kernels_decode.cu", "paper_2608_24204_gb300/csrc/common.cuh",
+KERNEL_SOURCES = ["paper_2608_24204_gb300/csrc/decode_step.cuh", "paper_2608_24204_gb300/csrc/gemv.cuh",
+                  "paper_2608_24204_gb300/csrc/kernels_decode.cu", "paper_2608_24204_gb300/csrc/common.cuh",
                   "paper_2608_24204_gb300/csrc/plan.h"]
 
 
@@ -533,18 +534,10 @@ def run_ours(args):
     model.prefill(prompt)
     n_prof = 8
     prof = wici.wici_profile_decode(model.ctx, n_prof)
-    if "decode_step" in prof:
-        # the persistent decode kernel: one launch streams the whole step
-        name = "decode_step"
-        unit_bytes = sum(gen.decode_bytes_per_token(CFG, PROMPT + i) for i in range(1, n_prof + 1)) / n_prof
-        traffic = profiled_traffic("decode_step_llama3-8b.md")
-    else:
-        # multi-launch decode (only for widths without a persistent instantiation;
-        # not the case at this shape): the gate/up GEMV is the largest launch
-        name = "gate_up_swiglu"
-        H, F = CFG.hidden, CFG.ffn_dim
-        unit_bytes = 2 * F * H * 2 + H * 2 + H * 4 + F * 4   # Wg|Wu + gain + x read + m written
-        traffic = None
+    # the persistent decode kernel: one launch streams the whole step
+    name = "decode_step"
+    unit_bytes = sum(gen.decode_bytes_per_token(CFG, PROMPT + i) for i in range(1, n_prof + 1)) / n_prof
+    traffic = profiled_traffic("decode_step_llama3-8b.md")
     n_k, ms_k = prof[name]
     k_gbs = unit_bytes / (ms_k / n_k / 1000.0) / 1e9
     roofline = {"bound": "hbm", "kernel": name, "achieved": k_gbs, "peak": pk["hbm_gbs"],

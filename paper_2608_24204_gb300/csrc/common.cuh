@@ -14,7 +14,6 @@ enum CtrlSlot : int {
     CTRL_ERR = 2,        // nonzero: a bounded wait gave up (site id)
     CTRL_LM_TICKET = 3,  // last-CTA ticket of the LM-head argmax
     CTRL_EPOCH = 4,      // persistent decode steps finished: names the tags of the next one
-    CTRL_ATTN_TICKET0 = 16,  // per KV head tickets of the flash-decode combine
     CTRL_WORDS = 128,
 };
 

@@ -17,13 +17,8 @@ struct Bufs {
     uint16_t *KV;     // paged KV pool (bf16 bits)
     int *ctrl;        // control words (CtrlSlot)
     int *hist;        // hist[p] = greedy token produced for position p   [max_tokens + 1]
-    float *x;         // decode residual stream                             [H]
-    float *q;         // decode query after RoPE                            [qdim]
-    float *o;         // decode attention output                            [qdim]
-    float *m;         // decode SwiGLU output                               [F]
     float *logits;    // last logits                                        [V]
     int2 *amax;       // per-CTA argmax partials (value bits, index)        [num_sms]
-    float *fd_part;   // flash-decode split states                           [nkv][splits][group][d + 4]
     uint32_t *mega_bound; // persistent decode: row-share boundaries (2^24 = all) [num_sms + 1]
     float *mega_time;     // persistent decode: gate/up time per CTA, last step (us) [num_sms]
     // persistent decode: words that carry a tag beside their value, all of them zero at first
@@ -78,11 +73,6 @@ struct LaunchHook {
     virtual ~LaunchHook() {}
 };
 
-// Flash-decode split count for a context of max_pages pages, and the floats
-// of its split-state buffer.
-int fd_splits(int max_pages);
-size_t fd_part_floats(int nkv, int group, int d, int max_pages);
-
 // Words of the persistent step's attention split states.
 size_t mega_part_words(int nkv, int group, int d);
 
@@ -96,13 +86,13 @@ cudaError_t enqueue_lm_head_argmax_raw(const uint16_t *W, const uint16_t *gain, 
                                        float eps, float *logits, int *ctrl, int2 *partials, int *hist, int grid,
                                        cudaStream_t st);
 
-// True when the decode step runs as one persistent kernel for this plan.
-bool decode_is_persistent(const Plan &p);
+// True when the plan's widths have a decode-step instantiation of their own (the 8-bit
+// format and the q/k norm need one; other bf16 widths run the one for any widths).
+bool decode_has_named_shape(const Plan &p);
 
 // Whole decode step for the token in ctrl[CTRL_TOKEN] at position ctrl[CTRL_POS]:
-// one persistent launch, or 5 launches per layer + the LM head (`pdl` enables programmatic
-// dependent launch between them).  map_kv: the KV pool's tensor map.
-cudaError_t enqueue_decode_step(const Plan &p, const Bufs &b, const CUtensorMap &map_kv, cudaStream_t st, bool pdl,
+// one persistent launch.  map_kv: the KV pool's tensor map.
+cudaError_t enqueue_decode_step(const Plan &p, const Bufs &b, const CUtensorMap &map_kv, cudaStream_t st,
                                 LaunchHook *hook);
 
 // Final RMSNorm + LM head + argmax of the row x [H]; the last CTA writes

@@ -45,8 +45,8 @@ struct Plan {
     size_t kv_layer_elems;  // max_pages pages
     size_t kv_elems;
     // workspace (byte offsets)
-    size_t ws_ctrl, ws_hist, ws_x, ws_q, ws_o, ws_m, ws_logits, ws_amax, ws_rope,
-        ws_pages, ws_tok, ws_X, ws_fd_part, ws_mega_bound, ws_mega_time;
+    size_t ws_ctrl, ws_hist, ws_logits, ws_amax, ws_rope,
+        ws_pages, ws_tok, ws_X, ws_mega_bound, ws_mega_time;
     size_t ws_tags, tag_bytes;   // the persistent decode step's tagged words
     size_t ws_Q[3], ws_A[3], ws_O[3], ws_M[3];   // one buffer per bf16 term
     size_t ws_Wt[3];        // 8-bit format only: one matrix dequantised as three bf16 terms (prefill)

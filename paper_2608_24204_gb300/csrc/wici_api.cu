@@ -135,13 +135,8 @@ const char *wici::make_plan(const wici_config *cfg, int num_sms, Plan *p) {
     const size_t T = (size_t)P.max_chunk;
     P.ws_ctrl = ws(CTRL_WORDS * sizeof(int));
     P.ws_hist = ws(((size_t)c.max_tokens + 1) * sizeof(int));
-    P.ws_x = ws(H * 4);
-    P.ws_q = ws((size_t)P.qdim * 4);
-    P.ws_o = ws((size_t)P.qdim * 4);
-    P.ws_m = ws(F * 4);
     P.ws_logits = ws(V * 4);
     P.ws_amax = ws((size_t)P.num_sms * sizeof(int2));
-    P.ws_fd_part = ws(fd_part_floats(P.nkv, P.group, P.d, P.max_pages) * sizeof(float));
     P.ws_mega_bound = ws(((size_t)P.num_sms + 1) * sizeof(uint32_t));
     P.ws_mega_time = ws((size_t)P.num_sms * sizeof(float));
     // tagged words (32-byte aligned arrays): q|k|v, residual after O and after down, o, m, split states
@@ -173,13 +168,8 @@ static Bufs make_bufs(const Plan &p, void *W, void *KV, void *WS) {
     b.KV = (uint16_t *)KV;
     b.ctrl = (int *)(ws + p.ws_ctrl);
     b.hist = (int *)(ws + p.ws_hist);
-    b.x = (float *)(ws + p.ws_x);
-    b.q = (float *)(ws + p.ws_q);
-    b.o = (float *)(ws + p.ws_o);
-    b.m = (float *)(ws + p.ws_m);
     b.logits = (float *)(ws + p.ws_logits);
     b.amax = (int2 *)(ws + p.ws_amax);
-    b.fd_part = (float *)(ws + p.ws_fd_part);
     b.mega_bound = (uint32_t *)(ws + p.ws_mega_bound);
     b.mega_time = (float *)(ws + p.ws_mega_time);
     b.tags = (uint64_t *)(ws + p.ws_tags);
@@ -317,13 +307,13 @@ int wici_create(const wici_config *cfg, void *cuda_stream, void *weight_dev, voi
         delete c;
         return fail(nullptr, WICI_E_ARG, "config: %s", m);
     }
-    if (c->plan.qk_norm && !decode_is_persistent(c->plan)) {
+    if (c->plan.qk_norm && !decode_has_named_shape(c->plan)) {
         delete c;
         return fail(nullptr, WICI_E_ARG,
                     "config: the per-head q/k norm is built into the one-launch decode step, which needs "
                     "n_q_heads * head_dim == hidden and an instantiated width");
     }
-    if (c->plan.q8 && !decode_is_persistent(c->plan)) {
+    if (c->plan.q8 && !decode_has_named_shape(c->plan)) {
         delete c;
         return fail(nullptr, WICI_E_ARG,
                     "config: the 8-bit block format is built for hidden 4096 / ffn 14336 (head_dim 128) and for "
@@ -550,7 +540,6 @@ static int finish_call(wici_ctx *c, int32_t new_kv_len, int32_t *token_out) {
         cudaMemsetAsync(c->bufs.ctrl + CTRL_LM_TICKET, 0, sizeof(int), c->stream);
         // the step that gave up is run again under the same tags: none of its words may stay
         cudaMemsetAsync(c->bufs.tags, 0, c->plan.tag_bytes, c->stream);
-        cudaMemsetAsync(c->bufs.ctrl + CTRL_ATTN_TICKET0, 0, 64 * sizeof(int), c->stream);
         cudaStreamSynchronize(c->stream);
         return fail(c, WICI_E_TIMEOUT, "a device-side wait gave up (site %d)", errw);
     }
@@ -590,7 +579,7 @@ static int ensure_graph(wici_ctx *c) {
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        cudaError_t e2 = enqueue_decode_step(c->plan, c->bufs, c->maps.kv, cap, true, nullptr);
+        cudaError_t e2 = enqueue_decode_step(c->plan, c->bufs, c->maps.kv, cap, nullptr);
         e = cudaStreamEndCapture(cap, &g);
         if (e2 != cudaSuccess) e = e2;
     }
@@ -631,10 +620,10 @@ static int begin_decode(wici_ctx *c, int32_t n_steps, int32_t token_in) {
 constexpr int kShareDepth = 2;
 
 static cudaError_t launch_step(wici_ctx *c) {
-    if (c->plan.cfg.max_sms > 0 && decode_is_persistent(c->plan)) {
+    if (c->plan.cfg.max_sms > 0) {
         cudaEvent_t ev = c->step_done[c->steps_launched % kShareDepth];
         cudaError_t e = c->steps_launched >= kShareDepth ? cudaEventSynchronize(ev) : cudaSuccess;
-        if (e == cudaSuccess) e = enqueue_decode_step(c->plan, c->bufs, c->maps.kv, c->stream, false, nullptr);
+        if (e == cudaSuccess) e = enqueue_decode_step(c->plan, c->bufs, c->maps.kv, c->stream, nullptr);
         if (e == cudaSuccess) e = cudaEventRecord(ev, c->stream);
         if (e == cudaSuccess) ++c->steps_launched;
         return e;
@@ -755,7 +744,7 @@ int wici_profile_decode(wici_ctx *c, int32_t n_steps, const char **names, int32_
     EventHook hook;
     hook.st = c->stream;
     for (int i = 0; i < n_steps; ++i) {
-        cudaError_t e = enqueue_decode_step(c->plan, c->bufs, c->maps.kv, c->stream, false, &hook);
+        cudaError_t e = enqueue_decode_step(c->plan, c->bufs, c->maps.kv, c->stream, &hook);
         if (e != cudaSuccess) return fail(c, WICI_E_CUDA, "profile launch: %s", cudaGetErrorString(e));
     }
     int rc = finish_call(c, c->kv_len + n_steps, nullptr);
