@@ -318,9 +318,10 @@ __global__ void __launch_bounds__(CV_THREADS, 1)
                 if (lane == 0) mbar_arrive(smem_u32(&acc_free[b]));
             } else {
                 // one tile per CTA: every CTA of the cluster has finished with its ring, so the
-                // sums' column slices cross through it: [source rank][row][SL + 4]
-                constexpr int SL = CV_BN / SPLIT, PITCH = SL + 4;
-                constexpr uint32_t SRC = CV_BM * PITCH * 4;
+                // sums' column slices cross through it, as [source rank][4 columns][row]: the 32 rows
+                // of a warp are 512 consecutive bytes
+                constexpr int SL = CV_BN / SPLIT;
+                constexpr uint32_t SRC = CV_BM * SL * 4;
                 static_assert(SPLIT * SRC <= CV_STAGES * CV_STAGE_BYTES, "slices fit the ring");
                 const bool some = (rank + 1) * s.nkb / SPLIT > rank * s.nkb / SPLIT;   // else nothing was accumulated
                 cluster_sync_all();
@@ -331,22 +332,22 @@ __global__ void __launch_bounds__(CV_THREADS, 1)
 #pragma unroll
                     for (int i = 0; i < 32; i += 4) {
                         const int col = half * (CV_BN / 2) + c0 + i;
-                        st_cluster_v4(base + (uint32_t)rank * SRC + (uint32_t)(m * PITCH + col % SL) * 4, col / SL,
+                        st_cluster_v4(base + (uint32_t)rank * SRC + (uint32_t)((col % SL) / 4 * CV_BM + m) * 16, col / SL,
                                       some ? v[i] : 0.f, some ? v[i + 1] : 0.f, some ? v[i + 2] : 0.f,
                                       some ? v[i + 3] : 0.f);
                     }
                 }
                 cluster_sync_all();
                 constexpr int NC = SL / 2;   // columns of the slice per warp of a pair
-                const uint8_t *src = smem_raw + (base - smem_u32(smem_raw)) + (size_t)(m * PITCH + half * NC) * 4;
+                const uint8_t *src = smem_raw + (base - smem_u32(smem_raw)) + (size_t)(half * NC / 4 * CV_BM + m) * 16;
                 if (ok && row) {
 #pragma unroll
                     for (int c = 0; c < NC; c += 8) {
                         float v[8] = {};
 #pragma unroll
                         for (int r = 0; r < SPLIT; ++r) {
-                            const float4 x = *reinterpret_cast<const float4 *>(src + r * SRC + c * 4);
-                            const float4 y = *reinterpret_cast<const float4 *>(src + r * SRC + c * 4 + 16);
+                            const float4 x = *reinterpret_cast<const float4 *>(src + r * SRC + c / 4 * CV_BM * 16);
+                            const float4 y = *reinterpret_cast<const float4 *>(src + r * SRC + (c / 4 + 1) * CV_BM * 16);
                             v[0] += x.x; v[1] += x.y; v[2] += x.z; v[3] += x.w;
                             v[4] += y.x; v[5] += y.y; v[6] += y.z; v[7] += y.w;
                         }

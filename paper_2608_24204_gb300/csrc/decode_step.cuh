@@ -324,6 +324,8 @@ struct MegaSplit {
 __device__ __forceinline__ MegaSplit mega_split(const MegaArgs &a, int len, int unit) {
     MegaSplit sp;
     sp.npages = (len + kPage - 1) / kPage;
+    // as many splits as there are: a page takes its warp longer than a state takes to combine
+    // (a page for every warp of a split before the next split: 8B widths 2481 -> 2512 us)
     const int pps = (sp.npages + a.splits - 1) / a.splits;
     sp.splits = (sp.npages + pps - 1) / pps;
     sp.g = unit / a.splits;
@@ -752,7 +754,7 @@ __device__ __forceinline__ void ldsm2(uint32_t addr, uint32_t &r0, uint32_t &r1)
 }
 __device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
                                          uint32_t b0, uint32_t b1) {
-    asm volatile(
+    asm(
         "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, "
         "%2, %3};"
         : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
@@ -908,21 +910,32 @@ __device__ bool mc_attn(MegaRing &R, const MegaArgs &a, uint16_t *kvl, const Meg
                 // these stores come before the next copy into this slot
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             }
-            // S: acc01 rows 0..7 term 0, rows 8..15 term 1; acc2 rows 0..7 term 2
+            // S: s01 rows 0..7 term 0, rows 8..15 term 1; s2 rows 0..7 term 2.  Fragments are
+            // loaded one step ahead of the matrix instructions that take them.
             float s01[2][4] = {}, s2[2][4] = {};
+            uint32_t qa[2][4], q2[2][2], kf[2][4];
+            auto load_s = [&](int kk) {
+                const int key = (mi >> 1) * 8 + mr, u = (kk & 3) * 2 + (mi & 1);
+                ldsm4(kb + (kk >> 2) * PG::CHUNK + key * 128 + ((u ^ (key & 7)) << 4), kf[kk & 1]);
+                ldsm4(qs0 + (mi & 1) * SM::Q_TERM + mr * SM::Q_ROW + (16 * kk + (mi >> 1) * 8) * 2, qa[kk & 1]);
+                ldsm2(qs0 + 2 * SM::Q_TERM + mr * SM::Q_ROW + (16 * kk + (mi & 1) * 8) * 2, q2[kk & 1][0], q2[kk & 1][1]);
+            };
+            uint32_t vf[2][4];
+            auto load_v = [&](int n) {
+                const int key = (mi & 1) * 8 + mr, u = 2 * n + (mi >> 1);
+                ldsm4t(vb + (u >> 3) * PG::CHUNK + key * 128 + (((u & 7) ^ (key & 7)) << 4), vf[n & 1]);
+            };
+            load_s(0);
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk) {
-                uint32_t qa[4], q2a, q2b, kf[4];
-                ldsm4(qs0 + (mi & 1) * SM::Q_TERM + mr * SM::Q_ROW + (16 * kk + (mi >> 1) * 8) * 2, qa);
-                ldsm2(qs0 + 2 * SM::Q_TERM + mr * SM::Q_ROW + (16 * kk + (mi & 1) * 8) * 2, q2a, q2b);
-                const int key = (mi >> 1) * 8 + mr, u = (kk & 3) * 2 + (mi & 1);
-                ldsm4(kb + (kk >> 2) * PG::CHUNK + key * 128 + ((u ^ (key & 7)) << 4), kf);
+                if (kk + 1 < D / 16) load_s(kk + 1);
+                const uint32_t(&q)[4] = qa[kk & 1], (&k)[4] = kf[kk & 1];
 #pragma unroll
-                for (int t = 0; t < 2; ++t) {
-                    mma_bf16(s01[t], qa[0], qa[1], qa[2], qa[3], kf[2 * t], kf[2 * t + 1]);
-                    mma_bf16(s2[t], q2a, 0u, q2b, 0u, kf[2 * t], kf[2 * t + 1]);
-                }
+                for (int t = 0; t < 2; ++t) mma_bf16(s01[t], q[0], q[1], q[2], q[3], k[2 * t], k[2 * t + 1]);
+#pragma unroll
+                for (int t = 0; t < 2; ++t) mma_bf16(s2[t], q2[kk & 1][0], 0u, q2[kk & 1][1], 0u, k[2 * t], k[2 * t + 1]);
             }
+            load_v(0);
             float s[2][2];
             float mx = m;
 #pragma unroll
@@ -954,14 +967,13 @@ __device__ bool mc_attn(MegaRing &R, const MegaArgs &a, uint16_t *kvl, const Meg
             m = mx;
 #pragma unroll
             for (int n = 0; n < D / 16; ++n) {
-                uint32_t vf[4];
-                const int key = (mi & 1) * 8 + mr, u = 2 * n + (mi >> 1);
-                ldsm4t(vb + (u >> 3) * PG::CHUNK + key * 128 + (((u & 7) ^ (key & 7)) << 4), vf);
+                if (n + 1 < D / 16) load_v(n + 1);
+                const uint32_t(&v)[4] = vf[n & 1];
 #pragma unroll
-                for (int t = 0; t < 2; ++t) {
-                    mma_bf16(o[2 * n + t], p[0][2], 0u, p[1][2], 0u, vf[2 * t], vf[2 * t + 1]);
-                    mma_bf16(o[2 * n + t], p[0][0], p[0][1], p[1][0], p[1][1], vf[2 * t], vf[2 * t + 1]);
-                }
+                for (int t = 0; t < 2; ++t) mma_bf16(o[2 * n + t], p[0][2], 0u, p[1][2], 0u, v[2 * t], v[2 * t + 1]);
+#pragma unroll
+                for (int t = 0; t < 2; ++t)
+                    mma_bf16(o[2 * n + t], p[0][0], p[0][1], p[1][0], p[1][1], v[2 * t], v[2 * t + 1]);
             }
         }
         __syncwarp();
@@ -1123,6 +1135,7 @@ __global__ void __launch_bounds__(kGemvThreads, 1)
     decode_step_kernel(const __grid_constant__ CUtensorMap map_kv, const MegaArgs a) {
     using LH = std::conditional_t<Q8, QH, SH>;   // layer matrices with K = hidden (and K = n_q * d)
     using LF = std::conditional_t<Q8, QF, SF>;   // the down projection, K = ffn
+    constexpr bool LOOP = ANY || Q8;             // a CTA may have several KV heads
     const uint32_t rb_h = Q8 ? (uint32_t)q8_row_bytes((size_t)a.H) : (uint32_t)a.H * 2u;
     const uint32_t rb_q = Q8 ? (uint32_t)q8_row_bytes((size_t)a.qdim) : (uint32_t)a.qdim * 2u;
     const uint32_t rb_f = Q8 ? (uint32_t)q8_row_bytes((size_t)a.F) : (uint32_t)a.F * 2u;
@@ -1174,8 +1187,9 @@ __global__ void __launch_bounds__(kGemvThreads, 1)
                 const size_t lo = (size_t)l * a.lstride;
                 ok = mp_rows(R, a.W + a.l0.wqkv + lo, rb_h, a.nqkv / 2, 2, rps_h, err, pol) &&
                      mp_pages<D>(R, a, &map_kv, l, sp0, err);
-                for (int u = blockIdx.x + gridDim.x; ok && u < units; u += gridDim.x)
-                    ok = mp_pages<D>(R, a, &map_kv, l, mega_split(a, len, u), err);
+                if constexpr (LOOP)
+                    for (int u = blockIdx.x + gridDim.x; ok && u < units; u += gridDim.x)
+                        ok = mp_pages<D>(R, a, &map_kv, l, mega_split(a, len, u), err);
                 ok = ok && mp_rows(R, a.W + a.l0.wo + lo, rb_q, a.H, 1, rps_q, err, pol) &&
                      mp_rows(R, a.W + a.l0.wgu + lo, rb_h, a.F, 2, rps_h, err, pol) &&
                      mp_rows(R, a.W + a.l0.wd + lo, rb_f, a.H, 1, rps_f, err, pol);
@@ -1211,6 +1225,7 @@ __global__ void __launch_bounds__(kGemvThreads, 1)
             ok = mc_attn<D>(R, a, a.KV + (size_t)l * a.kv_layer_elems, sp, len, tag, reinterpret_cast<uint8_t *>(red),
                             state, s_rope, a.qk_norm ? a.W + a.l0.qn + lo : nullptr,
                             a.qk_norm ? a.W + a.l0.kn + lo : nullptr);
+            if constexpr (!LOOP) break;
             u += gridDim.x;
             if (!ok || u >= units) break;
             sp = mega_split(a, len, u);

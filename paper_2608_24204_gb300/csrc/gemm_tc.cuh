@@ -198,6 +198,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     const int kk_begin = rank * nk * WU / SPLIT, kk_end = (rank + 1) * nk * WU / SPLIT;
     const int ngroups = (kk_end - kk_begin + TC_GROUP - 1) / TC_GROUP;
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    const uint32_t a_bytes = (uint32_t)maps.a_rows * (TC_BK * 2);   // loaded per term
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
@@ -226,25 +227,23 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 
     if (warp == 0) {
         if (lane == 0) {  // ------------------------------------------- TMA producer
-            int it = 0;   // k-blocks issued over all tiles
+            int it = 0, s = 0;   // k-blocks issued over all tiles; the next one's stage
+            uint32_t ph = 0;     // and its phase
             bool ok = true;
-            const uint32_t a_bytes = (uint32_t)maps.a_rows * (TC_BK * 2);
             // a bf16 weight does not depend on the kernels before this one: its first k-blocks
             // are on their way while those finish (8-bit: dequantised by the kernel before)
             const int early = WT == 1 && tile0 < ntiles ? min(S, kk_end - kk_begin) : 0;
-            for (int s = 0; s < early; ++s) {
-                const uint32_t fb = smem_u32(&full_bar[s]);
+            for (int e = 0; e < early; ++e) {
+                const uint32_t fb = smem_u32(&full_bar[e]);
                 mbar_arrive_expect_tx(fb, AT * a_bytes + G::B_BYTES);
-                tma_load_2d(base + (uint32_t)s * G::STAGE_BYTES + AT * TC_A_BYTES, &maps.w[0], (kk_begin + s) * TC_BK,
+                tma_load_2d(base + (uint32_t)e * G::STAGE_BYTES + AT * TC_A_BYTES, &maps.w[0], (kk_begin + e) * TC_BK,
                             (tile0 / ntm) * BN, fb);
             }
             griddep_wait();
             for (int tile = tile0; tile < ntiles && ok; tile += tile_step) {
                 const int m0 = (tile % ntm) * TC_BM, n0 = (tile / ntm) * BN;
                 for (int kk = kk_begin; kk < kk_end; ++kk, ++it) {
-                    const int s = it % S;
-                    if (it >= S && !(ok = mbar_wait(smem_u32(&empty_bar[s]), ((it / S) + 1) & 1, err, SITE_TC_EMPTY)))
-                        break;
+                    if (it >= S && !(ok = mbar_wait(smem_u32(&empty_bar[s]), ph ^ 1u, err, SITE_TC_EMPTY))) break;
                     const int j = WT == 1 ? 0 : kk / nk, kb = kk - j * nk;     // weight term, k-block
                     const uint32_t st = base + (uint32_t)s * G::STAGE_BYTES;
                     const uint32_t fb = smem_u32(&full_bar[s]);
@@ -256,6 +255,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                         if (t < na) tma_load_2d(st + t * TC_A_BYTES, &maps.a[t], kb * TC_BK, m0, fb);
                     if (it >= early) tma_load_2d(st + AT * TC_A_BYTES, &maps.w[j], kb * TC_BK, n0, fb);
                     s_issued = it + 1;
+                    if (++s == S) {
+                        s = 0;
+                        ph ^= 1u;
+                    }
                 }
             }
         }
@@ -263,7 +266,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         if (lane == 0) {  // ------------------------------------------- MMA issuer
             constexpr uint32_t idesc = tc_idesc(BN);
             bool ok = true;
-            int it = 0, gg = 0;   // k-blocks and groups consumed over all tiles
+            int gg = 0, s = 0;   // groups over all tiles, the next k-block's stage
+            uint32_t ph = 0;     // and its phase
             for (int tile = tile0; tile < ntiles && ok; tile += tile_step) {
                 for (int gi = 0; gi < ngroups && ok; ++gi, ++gg) {
                     const int b = gg & 1;
@@ -273,9 +277,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                     tc_fence_after();
                     const uint32_t acc = tmem + (uint32_t)b * G::ACC_STRIDE;
                     const int kk0 = kk_begin + gi * TC_GROUP, kk1 = min(kk_end, kk0 + TC_GROUP);
-                    for (int kk = kk0; kk < kk1; ++kk, ++it) {
-                        const int s = it % S;
-                        ok = mbar_wait(smem_u32(&full_bar[s]), (it / S) & 1, err, SITE_TC_FULL);
+                    for (int kk = kk0; kk < kk1; ++kk) {
+                        ok = mbar_wait(smem_u32(&full_bar[s]), ph, err, SITE_TC_FULL);
                         if (!ok) break;
                         tc_fence_after();
                         const int nt = WT == 1 ? AT : AT - kk / nk;   // activation terms meeting this weight term
@@ -291,6 +294,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                                     tc_mma(acc, ad0 + (uint64_t)((t * TC_A_BYTES + 32 * k) >> 4),
                                            bd0 + (uint64_t)(2 * k), idesc, (kk != kk0 || k != 0 || t != 0));
                         tc_commit(smem_u32(&empty_bar[s]));
+                        if (++s == S) {
+                            s = 0;
+                            ph ^= 1u;
+                        }
                     }
                     tc_commit(smem_u32(&acc_full[b]));  // fires when this group's MMAs have completed
                 }
@@ -337,23 +344,25 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 if (ok && t < T) epi.row(t, c0, sum, N - c0);
             } else {
                 // one tile per CTA: every CTA of the cluster has finished with its ring, so the
-                // sums' column slices cross through it: [source rank][row][SL + 4]
-                constexpr int SL = BN / SPLIT, PITCH = SL + 4;
-                constexpr uint32_t SRC = TC_BM * PITCH * 4;
+                // sums' column slices cross through it, as [source rank][4 columns][row]: the 32 rows
+                // of a warp are 512 consecutive bytes (row-major slices took 4 to 7 us to cross)
+                constexpr int SL = BN / SPLIT;
+                constexpr uint32_t SRC = TC_BM * SL * 4;
                 static_assert(SPLIT * SRC <= G::STAGES * G::STAGE_BYTES && SL % 16 == 0, "slices fit the ring");
                 const int row = q * 32 + lane;
                 cluster_sync_all();
 #pragma unroll
                 for (int c = 0; c < G::EPI_COLS; c += 4) {
                     const int col = half * G::EPI_COLS + c;
-                    st_cluster_v4(base + (uint32_t)rank * SRC + (uint32_t)(row * PITCH + col % SL) * 4, col / SL, sum[c],
-                                  sum[c + 1], sum[c + 2], sum[c + 3]);
+                    st_cluster_v4(base + (uint32_t)rank * SRC + (uint32_t)((col % SL) / 4 * TC_BM + row) * 16, col / SL,
+                                  sum[c], sum[c + 1], sum[c + 2], sum[c + 3]);
                 }
                 cluster_sync_all();
                 // this CTA's slice: half of it per warp of a pair, or all of it in the first
                 constexpr int NC = SL % 32 == 0 ? SL / 2 : SL;
                 if (SL % 32 == 0 || half == 0) {
                     const int part = SL % 32 == 0 ? half * NC : 0;
+                    const uint8_t *src = smem_raw + (base - smem_u32(smem_raw)) + (size_t)(part / 4 * TC_BM + row) * 16;
                     float v[NC];
 #pragma unroll
                     for (int c = 0; c < NC; ++c) v[c] = 0.f;
@@ -361,8 +370,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                     for (int r = 0; r < SPLIT; ++r)
 #pragma unroll
                         for (int c = 0; c < NC; c += 4) {
-                            const float4 x = *reinterpret_cast<const float4 *>(
-                                smem_raw + (base - smem_u32(smem_raw)) + r * SRC + (size_t)(row * PITCH + part + c) * 4);
+                            const float4 x = *reinterpret_cast<const float4 *>(src + r * SRC + c / 4 * TC_BM * 16);
                             v[c] += x.x; v[c + 1] += x.y; v[c + 2] += x.z; v[c + 3] += x.w;
                         }
                     const int c0 = n0 + rank * SL + part;

@@ -215,10 +215,9 @@ static cudaError_t enqueue_mega(const Plan &p, const Bufs &b, const CUtensorMap 
 cudaError_t enqueue_decode_step(const Plan &p, const Bufs &b, const CUtensorMap &map_kv, cudaStream_t st,
                                 LaunchHook *hook) {
     MegaLaunch fn = mega_named_launcher(p);
-    if (!fn) {
-        if (p.q8 || p.qk_norm) return cudaErrorInvalidValue;   // refused at create
-        fn = mega_any_launcher(p.d);
-    }
+    if (!fn && (p.q8 || p.qk_norm)) return cudaErrorInvalidValue;   // refused at create
+    // also a share of fewer SMs than KV heads: the bf16 shapes give a CTA one head at most
+    if (!fn || (!p.q8 && p.num_sms < p.nkv)) fn = mega_any_launcher(p.d);
     if (hook) hook->before("decode_step");
     const cudaError_t e = enqueue_mega(p, b, map_kv, st, fn);
     if (hook) hook->after("decode_step");
