@@ -40,6 +40,12 @@
 // the CTAs exchange column slices of their sums through shared memory (every CTA
 // adds the slices of its BN / SPLIT columns in rank order) and run the epilogue on
 // their slices.
+//
+// Chunks of at most 64 tokens (STACK, two activation terms): the two terms of the 64 rows
+// are the 128 rows of one tile, so each weight k-step is read by one MMA instead of two
+// (shared-memory ports bound these, too: 96 KB a k-block of 128 columns, 64 KB stacked).
+// Rows r and r + 64 of the accumulator are the two terms' sums; they meet in shared
+// memory on the way to the epilogue.
 // Every mbarrier wait is bounded; a wait that gives up records its site in
 // *err and the CTA still drains its copies, frees TMEM and exits.
 #pragma once
@@ -58,7 +64,7 @@ constexpr uint32_t TC_TMEM_COLS = 512;                                  // two a
 constexpr size_t TC_SMEM_BUDGET = 216 * 1024;                           // ring bytes
 
 // geometry of a 128 x BN output tile whose stages hold AT activation terms
-template <int BN, int AT = kTerms>
+template <int BN, int AT = kTerms>   // AT: 128-row blocks of activations per stage
 struct TcTile {
     static_assert(BN % 32 == 0 && BN <= 256, "BN: a multiple of 32 up to 256");
     static constexpr uint32_t B_BYTES = BN * TC_BK * 2;
@@ -171,16 +177,28 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, float *v) {
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// the epilogue warps of a cluster's CTAs (and their other warps), or those of a CTA by itself
+template <int SPLIT>
+__device__ __forceinline__ void exchange_sync() {
+    if constexpr (SPLIT > 1)
+        cluster_sync_all();
+    else
+        asm volatile("bar.sync 2, 256;" ::: "memory");
+}
+
 // Epi::row(t, c, v, n): output row t, the thread's span of columns from c on, of
 // which n are inside the matrix
-template <int BN, int SPLIT, int WT, class Epi>
+template <int BN, int SPLIT, bool STACK, int WT, class Epi>
 __global__ void __launch_bounds__(TC_THREADS, 1)
     gemm_tc_kernel(const __grid_constant__ GemmMaps maps, int T, int N, int K, int *err, const Epi epi) {
     static_assert(WT == 1 || WT == kTerms, "one exact bf16 weight term, or three");
     static_assert(SPLIT == 1 || SPLIT == 2 || SPLIT == 4, "CTAs of a tile");
     constexpr int AT = Epi::kATerms;   // activation terms multiplied (and loaded)
     static_assert(AT >= 1 && AT <= kTerms, "activation terms");
-    using G = TcTile<BN, AT>;
+    static_assert(!STACK || AT == 2, "two terms stacked");
+    using G = TcTile<BN, STACK ? 1 : AT>;
+    constexpr uint32_t A_TERM = STACK ? TC_A_BYTES / 2 : TC_A_BYTES;   // stacked: boxes of 64 rows
+    constexpr uint32_t A_STAGE = STACK ? TC_A_BYTES : AT * TC_A_BYTES;
     constexpr int S = G::STAGES;
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[S], empty_bar[S], acc_full[2], acc_free[2];
@@ -236,7 +254,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             for (int e = 0; e < early; ++e) {
                 const uint32_t fb = smem_u32(&full_bar[e]);
                 mbar_arrive_expect_tx(fb, AT * a_bytes + G::B_BYTES);
-                tma_load_2d(base + (uint32_t)e * G::STAGE_BYTES + AT * TC_A_BYTES, &maps.w[0], (kk_begin + e) * TC_BK,
+                tma_load_2d(base + (uint32_t)e * G::STAGE_BYTES + A_STAGE, &maps.w[0], (kk_begin + e) * TC_BK,
                             (tile0 / ntm) * BN, fb);
             }
             griddep_wait();
@@ -248,12 +266,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                     const uint32_t st = base + (uint32_t)s * G::STAGE_BYTES;
                     const uint32_t fb = smem_u32(&full_bar[s]);
                     // term j meets the activation terms i <= 2 - j only
-                    const int na = AT - j;
+                    const int na = STACK ? AT : AT - j;   // stacked: both terms, their MMAs are one
                     if (it >= early) mbar_arrive_expect_tx(fb, (uint32_t)na * a_bytes + G::B_BYTES);
 #pragma unroll
                     for (int t = 0; t < AT; ++t)
-                        if (t < na) tma_load_2d(st + t * TC_A_BYTES, &maps.a[t], kb * TC_BK, m0, fb);
-                    if (it >= early) tma_load_2d(st + AT * TC_A_BYTES, &maps.w[j], kb * TC_BK, n0, fb);
+                        if (t < na) tma_load_2d(st + t * A_TERM, &maps.a[t], kb * TC_BK, m0, fb);
+                    if (it >= early) tma_load_2d(st + A_STAGE, &maps.w[j], kb * TC_BK, n0, fb);
                     s_issued = it + 1;
                     if (++s == S) {
                         s = 0;
@@ -281,10 +299,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                         ok = mbar_wait(smem_u32(&full_bar[s]), ph, err, SITE_TC_FULL);
                         if (!ok) break;
                         tc_fence_after();
-                        const int nt = WT == 1 ? AT : AT - kk / nk;   // activation terms meeting this weight term
+                        const int nt = STACK ? 1 : WT == 1 ? AT : AT - kk / nk;   // activation terms meeting this weight term
                         const uint32_t st = base + (uint32_t)s * G::STAGE_BYTES;
                         // descriptors of k-step 0; each k-step of 16 elements is 32 bytes further
-                        const uint64_t bd0 = tc_desc_sw128(st + AT * TC_A_BYTES);
+                        const uint64_t bd0 = tc_desc_sw128(st + A_STAGE);
                         const uint64_t ad0 = tc_desc_sw128(st);
 #pragma unroll
                         for (int k = 0; k < TC_BK / 16; ++k)
@@ -339,7 +357,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&acc_free[b]));
             }
-            if constexpr (SPLIT == 1) {
+            if constexpr (SPLIT == 1 && !STACK) {
                 const int c0 = n0 + half * G::EPI_COLS;
                 if (ok && t < T) epi.row(t, c0, sum, N - c0);
             } else {
@@ -350,17 +368,17 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 constexpr uint32_t SRC = TC_BM * SL * 4;
                 static_assert(SPLIT * SRC <= G::STAGES * G::STAGE_BYTES && SL % 16 == 0, "slices fit the ring");
                 const int row = q * 32 + lane;
-                cluster_sync_all();
+                exchange_sync<SPLIT>();
 #pragma unroll
                 for (int c = 0; c < G::EPI_COLS; c += 4) {
                     const int col = half * G::EPI_COLS + c;
                     st_cluster_v4(base + (uint32_t)rank * SRC + (uint32_t)((col % SL) / 4 * TC_BM + row) * 16, col / SL,
                                   sum[c], sum[c + 1], sum[c + 2], sum[c + 3]);
                 }
-                cluster_sync_all();
+                exchange_sync<SPLIT>();
                 // this CTA's slice: half of it per warp of a pair, or all of it in the first
                 constexpr int NC = SL % 32 == 0 ? SL / 2 : SL;
-                if (SL % 32 == 0 || half == 0) {
+                if ((SL % 32 == 0 || half == 0) && (!STACK || q < 2)) {   // stacked: 64 rows of output
                     const int part = SL % 32 == 0 ? half * NC : 0;
                     const uint8_t *src = smem_raw + (base - smem_u32(smem_raw)) + (size_t)(part / 4 * TC_BM + row) * 16;
                     float v[NC];
@@ -372,6 +390,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                         for (int c = 0; c < NC; c += 4) {
                             const float4 x = *reinterpret_cast<const float4 *>(src + r * SRC + c / 4 * TC_BM * 16);
                             v[c] += x.x; v[c + 1] += x.y; v[c + 2] += x.z; v[c + 3] += x.w;
+                            if constexpr (STACK) {   // the second term's sums
+                                const float4 y =
+                                    *reinterpret_cast<const float4 *>(src + r * SRC + (c / 4 * TC_BM + TC_BM / 2) * 16);
+                                v[c] += y.x; v[c + 1] += y.y; v[c + 2] += y.z; v[c + 3] += y.w;
+                            }
                         }
                     const int c0 = n0 + rank * SL + part;
                     if (ok && t < T && c0 < N) epi.row(t, c0, v, N - c0);

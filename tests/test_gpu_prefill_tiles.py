@@ -1,5 +1,6 @@
 """Prefill GEMMs over the tile shapes their rule picks for short and ragged chunks:
-tiles shared by two and four CTAs, activation boxes of 32 to 96 rows, pairs of CTAs on
+tiles shared by two and four CTAs, activation boxes of 32 to 96 rows, both terms of up to
+64 rows in one tile, pairs of CTAs on
 256-row tiles, a chunk that ends one token into a tile, and widths whose last tile is
 partly outside the matrix.  Against the fp64 oracle with the parity rules."""
 import pytest
@@ -25,6 +26,8 @@ RAGGED = gen.TINY.with_(name="ragged", hidden=512, n_q_heads=12, n_kv_heads=4, f
 @pytest.mark.parametrize("cfg,prompt,chunk,q8", [
     (W8B, 1, 2048, False),
     (W8B, 33, 2048, False),
+    (W8B, 64, 2048, False),      # the two terms stacked in one tile
+    (W8B, 65, 2048, False),
     (W8B, 96, 2048, False),
     (W8B, 97, 2048, False),
     (W8B, 129, 2048, False),
