@@ -270,8 +270,8 @@ struct MEpiArgmax : EpiArgmax {
 };
 
 // ----------------------------------------------------------- producer side --
-// The producer keeps about kMegaFlightBytes of copies in flight per SM (never
-// fewer than two slots), and lets landed slots fill the rest of the ring.  That is
+// The producer keeps at least kMegaFlightBytes of copies in flight per SM (and two
+// slots), and lets landed slots fill the rest of the ring.  That is
 // what the HBM needs (152 SMs x 64 KB over ~1.3 us); more only queues in the memory
 // system, in front of the words that the phases exchange: with the whole ring in
 // flight and 192 KB of gate/up rows per SM moved to L2 during the attention phase,
@@ -279,7 +279,7 @@ struct MEpiArgmax : EpiArgmax {
 // 2491 (1B: 589 against 555); one slot in flight starves the HBM (3136 us).
 constexpr uint32_t kMegaFlightBytes = 65536;
 __device__ __forceinline__ int mega_flight(uint32_t slot_bytes) {
-    return min(kMegaSlots, max(2, (int)(kMegaFlightBytes / slot_bytes)));
+    return min(kMegaSlots, max(2, (int)((kMegaFlightBytes + slot_bytes - 1) / slot_bytes)));
 }
 
 // wait until ring slot R.n is free and at most `flight` - 1 earlier copies are still landing
@@ -415,6 +415,7 @@ __device__ bool mc_gemv(MegaRing &R, float *red, int K, int n_units, int rpu, co
     const int total_rows = (u1 - u0) * rpu;
     const int nst = (total_rows + RPS - 1) / RPS;
     if (nst == 0) return true;   // no rows: the input is not read (see the exchange rule above)
+    [[maybe_unused]] const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
     const int nchunks = K >> 3;
     if (tid < u1 - u0) epi.prefetch(u0 + tid);
     uint4 gw[NCH];
@@ -476,29 +477,49 @@ __device__ bool mc_gemv(MegaRing &R, float *red, int K, int n_units, int rpu, co
              mbar_wait(R.full0 + 8 * slot, (R.n / kMegaSlots) & 1, err, SITE_MEGA_FULL);
         if (!ok) *R.abort = 1;
         float acc[RPS];
-#pragma unroll
-        for (int r = 0; r < RPS; ++r) acc[r] = 0.f;
         const uint32_t sb = R.data0 + (uint32_t)slot * kMegaSlotBytes + (uint32_t)tid * 16u;
-        if (!ok) {
-        } else if (rows == RPS) {
+        if constexpr (!FULL) {
+            // this thread's chunks of all RPS rows into registers (past the last row: old bytes of
+            // the ring; no row's sum meets another's, and those are dropped), then the slot is free:
+            // its next copy need not wait for the products (steps of hidden 3072 414 -> 375 us,
+            // Qwen2.5-14B widths 637 -> 609, the 8-bit format at Qwen3-8B widths 524 -> 468)
+            uint4 w[RPS][NCH];
 #pragma unroll
             for (int r = 0; r < RPS; ++r)
 #pragma unroll
                 for (int j = 0; j < NCH; ++j)
-                    if (j < NCH - 1 || tail_ok)
-                        acc[r] = dot8(lds128(sb + r * row_bytes + j * kGemvConsumers * 16), h[j], acc[r]);
-        } else {
+                    w[r][j] = j < NCH - 1 || tail_ok ? lds128(sb + r * row_bytes + j * kGemvConsumers * 16) : zero;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(R.empty0 + 8 * slot);
+            ++R.n;
 #pragma unroll
-            for (int r = 0; r < RPS; ++r)
-                if (r < rows)
+            for (int r = 0; r < RPS; ++r) {
+                acc[r] = 0.f;
+#pragma unroll
+                for (int j = 0; j < NCH; ++j) acc[r] = dot8(w[r][j], h[j], acc[r]);
+            }
+        } else {   // without tails, loads and products interleaved are better (1B widths 520 us against 540)
+#pragma unroll
+            for (int r = 0; r < RPS; ++r) acc[r] = 0.f;
+            if (!ok) {
+            } else if (rows == RPS) {
+#pragma unroll
+                for (int r = 0; r < RPS; ++r)
 #pragma unroll
                     for (int j = 0; j < NCH; ++j)
-                        if (j < NCH - 1 || tail_ok)
+                        acc[r] = dot8(lds128(sb + r * row_bytes + j * kGemvConsumers * 16), h[j], acc[r]);
+            } else {
+#pragma unroll
+                for (int r = 0; r < RPS; ++r)
+                    if (r < rows)
+#pragma unroll
+                        for (int j = 0; j < NCH; ++j)
                             acc[r] = dot8(lds128(sb + r * row_bytes + j * kGemvConsumers * 16), h[j], acc[r]);
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(R.empty0 + 8 * slot);
+            ++R.n;
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(R.empty0 + 8 * slot);
-        ++R.n;
         warp_rows_store<RPS>(acc, red + (size_t)(buf * kGemvWarps + warp) * kRedRows + brow, rows, lane);
         brow += rows;
         if (s == nst - 1 || brow + RPS > kRedRows) {
@@ -530,6 +551,7 @@ __device__ bool mc_gemv_q8(MegaRing &R, float *red, int K, int n_units, int rpu,
     const int total_rows = (u1 - u0) * rpu;
     const int nst = (total_rows + RPS - 1) / RPS;
     if (nst == 0) return true;   // no rows: the input is not read (see the exchange rule above)
+    [[maybe_unused]] const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
     const int nchunks = K >> 4;
     if (tid < u1 - u0) epi.prefetch(u0 + tid);
     uint4 gw[NCH][2];
@@ -641,40 +663,43 @@ __device__ bool mc_gemv_q8(MegaRing &R, float *red, int K, int n_units, int rpu,
         ok = ok && !*reinterpret_cast<volatile int *>(R.abort) &&
              mbar_wait(R.full0 + 8 * slot, (R.n / kMegaSlots) & 1, err, SITE_MEGA_FULL);
         if (!ok) *R.abort = 1;
-        float acc[RPS];
-#pragma unroll
-        for (int r = 0; r < RPS; ++r) acc[r] = 0.f;
-        // chunk c: codes at byte 16 c of the row, its block's scale at byte K + 2 (c / 2)
+        // as mc_gemv's shapes with tails; chunk c: codes at byte 16 c of the row, its block's scale at byte K + 2 (c / 2)
         const uint32_t s0 = R.data0 + (uint32_t)slot * kMegaSlotBytes;
-        const uint32_t sb = s0 + (uint32_t)tid * 16u;
-        const uint32_t sc = s0 + (uint32_t)K + (uint32_t)(tid >> 1) * 2u;
-        if (ok) {
+        const uint32_t sb = s0 + (uint32_t)tid * 16u, sc = s0 + (uint32_t)K + (uint32_t)(tid >> 1) * 2u;
+        uint4 w[RPS][NCH];
+        float d[RPS][NCH];
 #pragma unroll
-            for (int r = 0; r < RPS; ++r)
-                if (rows == RPS || r < rows)
+        for (int r = 0; r < RPS; ++r)
 #pragma unroll
-                    for (int j = 0; j < NCH; ++j)
-                        if (j < NCH - 1 || tail_ok) {
-                            const uint4 w = lds128(sb + r * row_bytes + j * kGemvConsumers * 16);
-                            const float d = lds_f16(sc + r * row_bytes + j * (kGemvConsumers / 2) * 2);
-                            const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
-                            int a[ND];
-#pragma unroll
-                            for (int i = 0; i < ND; ++i) a[i] = 0;
-#pragma unroll
-                            for (int k = 0; k < 4; ++k)
-#pragma unroll
-                                for (int i = 0; i < ND; ++i)
-                                    a[i] = i == 0 ? dp4a_ss(ws[k], dg[j][i][k], a[i]) : dp4a_su(ws[k], dg[j][i][k], a[i]);
-                            float cv = small_int_to_f32(a[0]);
-#pragma unroll
-                            for (int i = 1; i < ND; ++i) cv = fmaf(cv, 256.0f, small_int_to_f32(a[i]));
-                            acc[r] = fmaf(d, cv, acc[r]);
-                        }
-        }
+            for (int j = 0; j < NCH; ++j) {
+                const bool in = j < NCH - 1 || tail_ok;
+                w[r][j] = in ? lds128(sb + r * row_bytes + j * kGemvConsumers * 16) : zero;
+                d[r][j] = in ? lds_f16(sc + r * row_bytes + j * (kGemvConsumers / 2) * 2) : 0.f;
+            }
         __syncwarp();
         if (lane == 0) mbar_arrive(R.empty0 + 8 * slot);
         ++R.n;
+        float acc[RPS];
+#pragma unroll
+        for (int r = 0; r < RPS; ++r) {
+            acc[r] = 0.f;
+#pragma unroll
+            for (int j = 0; j < NCH; ++j) {
+                const uint32_t ws[4] = {w[r][j].x, w[r][j].y, w[r][j].z, w[r][j].w};
+                int a[ND];
+#pragma unroll
+                for (int i = 0; i < ND; ++i) a[i] = 0;
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+#pragma unroll
+                    for (int i = 0; i < ND; ++i)
+                        a[i] = i == 0 ? dp4a_ss(ws[k], dg[j][i][k], a[i]) : dp4a_su(ws[k], dg[j][i][k], a[i]);
+                float cv = small_int_to_f32(a[0]);
+#pragma unroll
+                for (int i = 1; i < ND; ++i) cv = fmaf(cv, 256.0f, small_int_to_f32(a[i]));
+                acc[r] = fmaf(d[r][j], cv, acc[r]);
+            }
+        }
         warp_rows_store<RPS>(acc, red + (size_t)(buf * kGemvWarps + warp) * kRedRows + brow, rows, lane);
         brow += rows;
         if (s == nst - 1 || brow + RPS > kRedRows) {

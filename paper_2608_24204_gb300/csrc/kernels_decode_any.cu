@@ -1,7 +1,7 @@
 // The decode step for widths without an instantiation of their own (bf16): the same
 // persistent kernel with each phase's shape picked at run time.  Such widths used to run
 // as five launches a layer and the LM head, 77 us a layer at hidden 3072, ffn 8192 (24
-// heads of 128), against 46 here and 30 of HBM time.
+// heads of 128), against 41 here and 30 of HBM time.
 #include "decode_step.cuh"
 
 namespace wici {
