@@ -40,21 +40,27 @@ struct Bufs {
     float *QKraw;
 };
 
-// A weight matrix (or one of its terms) as 2-D maps with the boxes of the GEMM's tiles:
-// the tile's columns, or half of them where a pair of CTAs shares it.
-constexpr int kWeightBoxes = 5;
-constexpr int kWeightBox[kWeightBoxes] = {96, 112, 128, 192, 224};
-struct WeightMaps {
-    CUtensorMap box[kWeightBoxes];
+// A row-major bf16 matrix as 2-D tensor maps, one per box height that the prefill GEMMs
+// copy (rows of a short chunk, a tile's columns, or half of them where a pair of CTAs
+// shares it).  A map is encoded when a GEMM first asks for it: a matrix is used with one
+// or two of them, and encoding all when the context was created added 1.5 ms to it.
+constexpr int kMapBoxes = 7;
+constexpr int kMapBox[kMapBoxes] = {32, 64, 96, 112, 128, 192, 224};
+struct MatrixMaps {
+    const void *ptr = nullptr;
+    int rows = 0, K = 0;
+    mutable bool ready[kMapBoxes] = {};
+    mutable CUtensorMap map[kMapBoxes];
 };
+// the map with boxes of `box` rows, or nullptr when it cannot be encoded
+const CUtensorMap *matrix_map(const MatrixMaps &m, int box);
 
-// TMA descriptors of the prefill GEMM operands (built once per context).
+// TMA descriptors of the prefill GEMM operands.
 struct PrefillMaps {
-    // GEMM activations [i]: boxes of 32 (i + 1) rows, for chunks shorter than a 128-row tile
-    CUtensorMap a[4][kTerms], o[4][kTerms], m[4][kTerms];
+    MatrixMaps a[kTerms], o[kTerms], m[kTerms];        // GEMM activations
     CUtensorMap kv;                                    // the whole KV pool: [page][K|V][kv_head][16][d]
-    std::vector<WeightMaps> wqkv, wo, wgu, wd;         // per layer weights
-    WeightMaps wt_qkv[kTerms], wt_o[kTerms], wt_gu[kTerms], wt_d[kTerms];  // 8-bit format: the dequantised terms
+    std::vector<MatrixMaps> wqkv, wo, wgu, wd;         // per layer weights
+    MatrixMaps wt_qkv[kTerms], wt_o[kTerms], wt_gu[kTerms], wt_d[kTerms];  // 8-bit format: the dequantised terms
     int sms, pairs, quads;   // CTAs, clusters of two and clusters of four that run at once
 };
 
@@ -63,7 +69,7 @@ struct PrefillMaps {
 bool encode_tiled(CUtensorMap *m, int rank, const void *ptr, const uint64_t *dims, const uint64_t *strides_bytes,
                   const uint32_t *box, const uint32_t *elem_strides);
 
-// Encodes every tensor map of `m`; returns an error message or nullptr.
+// Fills `m` and sets the prefill kernels' limits; returns an error message or nullptr.
 const char *make_prefill_maps(const Plan &p, const Bufs &b, PrefillMaps *m);
 
 // Called around every launch when profiling (eager mode).

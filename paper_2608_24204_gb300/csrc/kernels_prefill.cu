@@ -9,6 +9,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <mutex>
 #include <type_traits>
 
 #include "common.cuh"
@@ -234,10 +235,21 @@ static bool encode_2d(CUtensorMap *m, const void *ptr, int rows, int K, int box_
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-static bool encode_w(WeightMaps *m, const void *ptr, int rows, int K) {
-    bool ok = true;
-    for (int i = 0; i < kWeightBoxes; ++i) ok = ok && encode_2d(&m->box[i], ptr, rows, K, kWeightBox[i]);
-    return ok;
+const CUtensorMap *matrix_map(const MatrixMaps &m, int box) {
+    for (int i = 0; i < kMapBoxes; ++i) {
+        if (kMapBox[i] != box) continue;
+        if (!m.ready[i]) m.ready[i] = encode_2d(&m.map[i], m.ptr, m.rows, m.K, box);
+        return m.ready[i] ? &m.map[i] : nullptr;
+    }
+    return nullptr;
+}
+
+static MatrixMaps matrix(const void *ptr, int rows, int K) {
+    MatrixMaps m;
+    m.ptr = ptr;
+    m.rows = rows;
+    m.K = K;
+    return m;
 }
 
 // the KV pool of every layer as [page (layer-major)][K|V][kv head][16 slots][d]:
@@ -258,53 +270,52 @@ static bool encode_kv(CUtensorMap *m, const void *ptr, const Plan &p) {
 
 const char *make_prefill_maps(const Plan &p, const Bufs &b, PrefillMaps *m) {
     const int T = p.max_chunk;
-    bool ok = true;
-    for (int t = 0; t < kTerms; ++t)
-        for (int x = 0; x < 4; ++x) {
-            const int box = 32 * (x + 1);
-            ok = ok && encode_2d(&m->a[x][t], b.A[t], T, p.H, box) && encode_2d(&m->o[x][t], b.O[t], T, p.qdim, box) &&
-                 encode_2d(&m->m[x][t], b.M[t], T, p.F, box);
-        }
-    if (!ok) return "cuTensorMapEncodeTiled failed for an activation operand";
-    ok = encode_kv(&m->kv, b.KV, p);
-    if (!ok) return "cuTensorMapEncodeTiled failed for the attention operands";
-    if (p.q8) {
-        // the 8-bit format: every GEMM reads the one dequantised matrix in the workspace
-        for (int t = 0; t < kTerms; ++t) {
-            ok = encode_w(&m->wt_qkv[t], b.Wt[t], p.nqkv, p.H) && encode_w(&m->wt_o[t], b.Wt[t], p.H, p.qdim) &&
-                 encode_w(&m->wt_gu[t], b.Wt[t], 2 * p.F, p.H) && encode_w(&m->wt_d[t], b.Wt[t], p.H, p.F);
-            if (!ok) return "cuTensorMapEncodeTiled failed for a dequantised weight matrix";
+    for (int t = 0; t < kTerms; ++t) {
+        m->a[t] = matrix(b.A[t], T, p.H);
+        m->o[t] = matrix(b.O[t], T, p.qdim);
+        m->m[t] = matrix(b.M[t], T, p.F);
+        if (p.q8) {   // the 8-bit format: every GEMM reads the one dequantised matrix in the workspace
+            m->wt_qkv[t] = matrix(b.Wt[t], p.nqkv, p.H);
+            m->wt_o[t] = matrix(b.Wt[t], p.H, p.qdim);
+            m->wt_gu[t] = matrix(b.Wt[t], 2 * p.F, p.H);
+            m->wt_d[t] = matrix(b.Wt[t], p.H, p.F);
         }
     }
-    m->wqkv.resize(p.q8 ? 0 : p.L);
-    m->wo.resize(p.q8 ? 0 : p.L);
-    m->wgu.resize(p.q8 ? 0 : p.L);
-    m->wd.resize(p.q8 ? 0 : p.L);
+    if (!encode_kv(&m->kv, b.KV, p)) return "cuTensorMapEncodeTiled failed for the attention operands";
     for (int l = 0; l < (p.q8 ? 0 : p.L); ++l) {
         const LayerOffsets &lo = p.layer[l];
-        ok = encode_w(&m->wqkv[l], b.W + lo.wqkv, p.nqkv, p.H) && encode_w(&m->wo[l], b.W + lo.wo, p.H, p.qdim) &&
-             encode_w(&m->wgu[l], b.W + lo.wgu, 2 * p.F, p.H) && encode_w(&m->wd[l], b.W + lo.wd, p.H, p.F);
-        if (!ok) return "cuTensorMapEncodeTiled failed for a weight matrix";
+        m->wqkv.push_back(matrix(b.W + lo.wqkv, p.nqkv, p.H));
+        m->wo.push_back(matrix(b.W + lo.wo, p.H, p.qdim));
+        m->wgu.push_back(matrix(b.W + lo.wgu, 2 * p.F, p.H));
+        m->wd.push_back(matrix(b.W + lo.wd, p.H, p.F));
     }
-    static bool attrs = false;
-    if (!attrs) {
-        const auto attr = [](const void *f, int bytes) {
-            return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
-        };
-        if (setup_gemm<PEpiQKV>() != cudaSuccess || setup_gemm<PEpiResidual>() != cudaSuccess ||
-            setup_gemm<PEpiSwiGLU>() != cudaSuccess ||
-            cudaFuncSetAttribute(attn_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(AttnSmem<128>::TOTAL + 1024)) != cudaSuccess ||
-            cudaFuncSetAttribute(attn_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(AttnSmem<64>::TOTAL + 1024)) != cudaSuccess)
-            return "cannot raise the shared-memory limit of the tensor-core GEMM";
-        attrs = true;
-    }
-    // resident clusters of two (the pair kernel) and of four, within this context's SM share
     m->sms = p.num_sms;
-    if (resident_clusters<PEpiSwiGLU>(2, p.num_sms, &m->pairs) != cudaSuccess ||
-        resident_clusters<PEpiSwiGLU>(4, p.num_sms, &m->quads) != cudaSuccess)
-        return "cannot query the resident clusters of the tensor-core GEMM";
+    // kernel limits and resident clusters: once per device
+    static std::mutex mu;
+    static int dev_pairs[64] = {}, dev_quads[64] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return "no CUDA device";
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        if (dev_pairs[dev] == 0) {
+            const auto limit = [](const void *f, size_t bytes) {
+                return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
+            };
+            int pairs = 0, quads = 0;
+            if (setup_gemm<PEpiQKV>() != cudaSuccess || setup_gemm<PEpiResidual>() != cudaSuccess ||
+                setup_gemm<PEpiSwiGLU>() != cudaSuccess ||
+                !limit((const void *)attn_tc_kernel<128>, AttnSmem<128>::TOTAL + 1024) ||
+                !limit((const void *)attn_tc_kernel<64>, AttnSmem<64>::TOTAL + 1024))
+                return "cannot raise the shared-memory limits of the prefill kernels";
+            if (resident_clusters<PEpiSwiGLU>(2, &pairs) != cudaSuccess ||
+                resident_clusters<PEpiSwiGLU>(4, &quads) != cudaSuccess || pairs < 1)
+                return "cannot query the resident clusters of the tensor-core GEMM";
+            dev_pairs[dev] = pairs;
+            dev_quads[dev] = quads;
+        }
+        m->pairs = dev_pairs[dev] < p.num_sms / 2 ? dev_pairs[dev] : p.num_sms / 2;
+        m->quads = dev_quads[dev] < p.num_sms / 4 ? dev_quads[dev] : p.num_sms / 4;
+    }
     return nullptr;
 }
 
@@ -333,8 +344,8 @@ cudaError_t launch_attn_tc(const Plan &p, const Bufs &b, const PrefillMaps &mp, 
 // bf16: the layer's own matrix; 8-bit format: dequantise the layer's rows into
 // the workspace terms first (stream order makes the previous GEMM finish reading them)
 template <class Epi>
-static cudaError_t weight_operand(const Plan &p, const Bufs &b, const WeightMaps &bf16_map,
-                                  const WeightMaps *terms, const uint16_t *rows, int n_rows, int K, cudaStream_t st,
+static cudaError_t weight_operand(const Plan &p, const Bufs &b, const MatrixMaps &bf16_map,
+                                  const MatrixMaps *terms, const uint16_t *rows, int n_rows, int K, cudaStream_t st,
                                   LaunchHook *hook, WOperand *w) {
     if (!p.q8) {
         *w = WOperand{{&bf16_map, &bf16_map, &bf16_map}, 1};

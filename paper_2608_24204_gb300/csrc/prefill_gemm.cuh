@@ -292,7 +292,7 @@ struct PEpiSwiGLU {  // interleaved (gate, up) columns -> M[t][c/2] = silu(g) * 
 // --------------------------------------------------------------- launches ----
 // the weight operand of one GEMM: one exact bf16 matrix, or three terms
 struct WOperand {
-    const WeightMaps *w[kTerms];
+    const MatrixMaps *w[kTerms];
     int terms;
 };
 
@@ -324,20 +324,19 @@ cudaError_t launch_gemm_pair(int pairs, const GemmMaps &maps, int terms, int T, 
                          epi);
 }
 
-// a: the activation's maps with boxes of 32, 64, 96 and 128 rows
 template <class Epi>
-cudaError_t gemm(const Plan &p, const PrefillMaps &mp, const CUtensorMap (&a)[4][kTerms], const WOperand &w,
+cudaError_t gemm(const Plan &p, const PrefillMaps &mp, const MatrixMaps (&a)[kTerms], const WOperand &w,
                         int T, int N, int K, int *err, const Epi &epi, cudaStream_t st, LaunchHook *hook,
                         const char *name) {
     const TileChoice c = pick_tile(T, N, K, Epi::kATerms, w.terms == 1 ? 1 : Epi::kATerms, mp);
     GemmMaps maps;
     // rows of a tile past the chunk are not loaded; a stacked tile is two boxes of 64
-    const int box = c.stack ? 1 : T < TC_BM ? (T - 1) / 32 : 3;
-    maps.a_rows = 32 * (box + 1);
+    maps.a_rows = c.stack ? 64 : T < TC_BM ? (T + 31) / 32 * 32 : TC_BM;
     for (int t = 0; t < kTerms; ++t) {
-        maps.a[t] = a[box][t];
-        for (int i = 0; i < kWeightBoxes; ++i)
-            if (kWeightBox[i] == (c.pair ? c.bn / 2 : c.bn)) maps.w[t] = w.w[t]->box[i];
+        const CUtensorMap *ma = matrix_map(a[t], maps.a_rows), *mw = matrix_map(*w.w[t], c.pair ? c.bn / 2 : c.bn);
+        if (!ma || !mw) return cudaErrorInvalidValue;
+        maps.a[t] = *ma;
+        maps.w[t] = *mw;
     }
     if (hook) hook->before(name);
     cudaError_t e;
@@ -398,11 +397,11 @@ cudaError_t setup_gemm() {
     return e;
 }
 
-// clusters of `size` (2: the pair kernel) that run at once within a share of `sms` SMs
+// clusters of `size` (2: the pair kernel) that run at once on the current device
 template <class Epi>
-cudaError_t resident_clusters(int size, int sms, int *n) {
+cudaError_t resident_clusters(int size, int *n) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(size * sms));
+    cfg.gridDim = dim3((unsigned)(size * 1024));
     cfg.blockDim = dim3(TC_THREADS);
     cfg.dynamicSmemBytes = size == 2 ? TcPairTile<256, 2>::SMEM : TcTile<128, 2>::SMEM;
     cudaLaunchAttribute attr[1];
@@ -412,17 +411,15 @@ cudaError_t resident_clusters(int size, int sms, int *n) {
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = size == 2 ? cudaOccupancyMaxActiveClusters(n, gemm2_tc_kernel<256, 1, Epi>, &cfg)
-                                    : cudaOccupancyMaxActiveClusters(n, gemm_tc_kernel<128, 4, false, 1, Epi>, &cfg);
-    if (e == cudaSuccess && *n > sms / size) *n = sms / size;
-    return e;
+    return size == 2 ? cudaOccupancyMaxActiveClusters(n, gemm2_tc_kernel<256, 1, Epi>, &cfg)
+                     : cudaOccupancyMaxActiveClusters(n, gemm_tc_kernel<128, 4, false, 1, Epi>, &cfg);
 }
 
 #define WICI_GEMM_INSTANCE(EXTERN, Epi)                                                                               \
-    EXTERN template cudaError_t gemm<Epi>(const Plan &, const PrefillMaps &, const CUtensorMap (&)[4][kTerms],       \
+    EXTERN template cudaError_t gemm<Epi>(const Plan &, const PrefillMaps &, const MatrixMaps (&)[kTerms],       \
                                           const WOperand &, int, int, int, int *, const Epi &, cudaStream_t,         \
                                           LaunchHook *, const char *);                                               \
     EXTERN template cudaError_t setup_gemm<Epi>();                                                                   \
-    EXTERN template cudaError_t resident_clusters<Epi>(int, int, int *);
+    EXTERN template cudaError_t resident_clusters<Epi>(int, int *);
 
 }  // namespace wici
