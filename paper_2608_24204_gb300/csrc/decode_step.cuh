@@ -175,18 +175,6 @@ __device__ __forceinline__ bool mega_input(float (&h)[NCH][CW], const uint64_t *
     return ok;
 }
 
-// one word, polled
-__device__ __forceinline__ bool mega_word(const uint64_t *p, uint32_t tag, float *v, int *err) {
-    PollLimit lim;
-    uint64_t w = ld_tagged(p);
-    while (!has_tag(w, tag)) {
-        if (!lim.again(err)) return false;
-        w = ld_tagged(p);
-    }
-    *v = tagged_value(w);
-    return true;
-}
-
 // ------------------------------------------------------- decode epilogues --
 // unit(u, v): v[0..rpu) are the finished dot products of unit u's rows;
 // prefetch(u): this thread finishes unit u in the phase's first batch of rows, so
@@ -1150,13 +1138,31 @@ __device__ inline void mega_rebalance(const MegaArgs &a, float *scr) {
     }
 }
 
+// Registers: nine warps get 168 each, the register file's share of three warps on one SM
+// partition.  Where a thread holds two or more chunks of every hidden-wide row (bf16 rows of
+// more than 2048 elements in a named shape), the step is launched with twelve warps of 168
+// and the producer's warpgroup hands its own on: 384 x 168 = 128 x 104 + 256 x 200.  The
+// compiler then keeps more loads of a phase in flight: Llama-3-8B widths, 2 layers and
+// 6360 tokens of context, 180 us a step -> 176; 14B widths, 6 layers, 599 -> 580.  The other
+// shapes lose with it (1B 518 -> 536 us, 8-bit Qwen3-8B 9 layers 471 -> 482, widths picked
+// at run time 366 -> 370) and keep nine warps.  A producer of 24 and consumers of 240
+// measured the same (174 to 176, 579).
+template <class SH, bool Q8, bool ANY>
+struct MegaRegs {
+    static constexpr bool kSplit = !Q8 && !ANY && SH::NCH >= 2;
+    static constexpr int kThreads = kSplit ? 384 : kGemvThreads;
+    static constexpr int kProducer = 104, kConsumer = 200;
+    // above the launch's own registers the consumers would wait for ever: launch_mega checks
+    static constexpr int kNeeded = 128 * kProducer + 256 * kConsumer;
+};
+
 // SH, SF: GEMV shapes of K = hidden and K = ffn for bf16 rows; with Q8 the seven
 // per-layer matrices are in the 8-bit block format and stream with the shapes
 // QH, QF (16-element chunks, rows per slot sized for the shorter rows), while
 // the LM head stays bf16 (SH).  ANY: bf16 matrices of any widths the configuration
 // allows, the shape of each phase picked at run time (SH .. QF are ignored).
 template <int D, class SH, class SF, bool Q8, class QH, class QF, bool ANY>
-__global__ void __launch_bounds__(kGemvThreads, 1)
+__global__ void __launch_bounds__((MegaRegs<SH, Q8, ANY>::kThreads), 1)
     decode_step_kernel(const __grid_constant__ CUtensorMap map_kv, const MegaArgs a) {
     using LH = std::conditional_t<Q8, QH, SH>;   // layer matrices with K = hidden (and K = n_q * d)
     using LF = std::conditional_t<Q8, QF, SF>;   // the down projection, K = ffn
@@ -1204,8 +1210,10 @@ __global__ void __launch_bounds__(kGemvThreads, 1)
     const MegaSplit sp0 = mega_split(a, len, blockIdx.x);
     const int units = a.nkv * a.splits;
 
-    if (warp == kGemvWarps) {  // ------------------------------------ producer
-        if (lane == 0) {
+    using Regs = MegaRegs<SH, Q8, ANY>;
+    if (warp >= kGemvWarps) {  // ------------------------------------ producer
+        if constexpr (Regs::kSplit) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(Regs::kProducer));
+        if (warp == kGemvWarps && lane == 0) {
             const uint64_t pol = l2_evict_first();
             bool ok = true;
             for (int l = 0; l < a.L && ok; ++l) {
@@ -1228,6 +1236,7 @@ __global__ void __launch_bounds__(kGemvThreads, 1)
     }
 
     // ---------------------------------------------------------------- consumers
+    if constexpr (Regs::kSplit) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(Regs::kConsumer));
     const uint16_t *embed = a.W + a.w_embed + (size_t)a.ctrl[CTRL_TOKEN] * a.H;
     // tag of layer l: unique over the last 2^32 / L steps
     const uint32_t tag0 = (uint32_t)a.ctrl[CTRL_EPOCH] * (uint32_t)a.L;
@@ -1288,9 +1297,17 @@ typedef cudaError_t (*MegaLaunch)(const CUtensorMap &, const MegaArgs &, int gri
 
 template <int D, class SH, class SF, bool Q8, class QH, class QF, bool ANY>
 cudaError_t launch_mega(const CUtensorMap &map_kv, const MegaArgs &a, int grid, cudaStream_t st) {
+    using Regs = MegaRegs<SH, Q8, ANY>;
+    if constexpr (Regs::kSplit) {   // a property of the compiled kernel, asked once
+        static const int regs = [] {
+            cudaFuncAttributes fa = {};
+            return cudaFuncGetAttributes(&fa, decode_step_kernel<D, SH, SF, Q8, QH, QF, ANY>) == cudaSuccess ? fa.numRegs : 0;
+        }();
+        if (regs * Regs::kThreads < Regs::kNeeded) return cudaErrorLaunchOutOfResources;
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(kGemvThreads);
+    cfg.blockDim = dim3(Regs::kThreads);
     cfg.dynamicSmemBytes = kMegaSmem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
