@@ -15,7 +15,7 @@ namespace wici {
 // Exchange between CTAs: every vector one phase hands to the next (q|k|v, the
 // attention split states and output, the residual after O and after down, the
 // SwiGLU vector) is an array of 64-bit words, the fp32 value below a 32-bit tag
-// that names the layer of the step (mega_tag).  A consumer polls the words it
+// that names the layer of the step.  A consumer polls the words it
 // needs until they carry the tag; a word is written with one 64-bit store, so a
 // value is never seen without its tag and no fence, counter or grid barrier is
 // needed.  A grid barrier (store, fence, atomic, poll, then load) cost 1.0 to 2.2
@@ -30,7 +30,7 @@ namespace wici {
 // read of layer l's.
 //
 // Measured (per layer of a decode step, 8B widths at context ~1060, bf16): 79.9
-// us with five grid barriers a layer, 72 us now; at 1B widths 35.0 and 27.5 us.
+// us with five grid barriers a layer, 70 us now; at 1B widths 35.0 and 27.5 us.
 constexpr int kMegaSlots = 6;
 constexpr uint32_t kMegaSlotBytes = 32768;
 constexpr int kMegaMaxCtas = 256;               // grid size limit (one CTA per SM)
