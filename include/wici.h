@@ -66,8 +66,9 @@ typedef struct wici_config {
                                 head_dim with its own gain ("layers.<l>.q_norm" / ".k_norm",
                                 [1, head_dim]) before RoPE (the paper's models are Qwen3,
                                 Sec. 5.1, Tab. 1) */
-    int32_t max_sms;         /* SM share: the context's kernels use at most this many SMs
-                                (0: all).  Several contexts whose shares add up to at most
+    int32_t max_sms;         /* SM share: the decode step, the GEMMs and the LM head of the context
+                                use at most this many SMs (0: all); a prefill's attention and its
+                                short row-wise kernels take the SMs that are free.  Several contexts whose shares add up to at most
                                 the GPU's SM count decode concurrently, each on its own
                                 stream (Sec. 5.4, multiple clients; Sec. 7, task scheduling:
                                 the caller's stream priorities order the tenants). */

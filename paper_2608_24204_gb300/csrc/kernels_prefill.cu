@@ -169,7 +169,7 @@ static cudaError_t dequant_terms(const Plan &p, const Bufs &b, const uint16_t *W
     const int grid = (int)((n + 255) / 256 < 8 * p.num_sms ? (n + 255) / 256 : 8 * p.num_sms);
     if (hook) hook->before("prefill_q8_dequant");
     const cudaError_t e =
-        launch_kernel(q8_dequant_terms_kernel, dim3(grid), 256, 0, st, 1, true, reinterpret_cast<const uint8_t *>(W), rows,
+        launch_kernel(q8_dequant_terms_kernel, dim3(grid), 256, 0, st, 1, p.pdl, reinterpret_cast<const uint8_t *>(W), rows,
                       K, Terms{{b.Wt[0], b.Wt[1], b.Wt[2]}}, nterms);
     if (hook) hook->after("prefill_q8_dequant");
     return e;
@@ -337,8 +337,8 @@ cudaError_t launch_attn_tc(const Plan &p, const Bufs &b, const PrefillMaps &mp, 
     a.scale_log2 = 1.4426950408889634f / sqrtf((float)p.d);
     dim3 grid(((T + a.tpt - 1) / a.tpt) * p.nkv);
     if (p.d == 128)
-        return launch_kernel(attn_tc_kernel<128>, grid, AT_THREADS, AttnSmem<128>::TOTAL + 1024, st, 1, true, mp.kv, a);
-    return launch_kernel(attn_tc_kernel<64>, grid, AT_THREADS, AttnSmem<64>::TOTAL + 1024, st, 1, true, mp.kv, a);
+        return launch_kernel(attn_tc_kernel<128>, grid, AT_THREADS, AttnSmem<128>::TOTAL + 1024, st, 1, p.pdl, mp.kv, a);
+    return launch_kernel(attn_tc_kernel<64>, grid, AT_THREADS, AttnSmem<64>::TOTAL + 1024, st, 1, p.pdl, mp.kv, a);
 }
 
 // bf16: the layer's own matrix; 8-bit format: dequantise the layer's rows into
@@ -359,7 +359,7 @@ cudaError_t enqueue_prefill_chunk(const Plan &p, const Bufs &b, const PrefillMap
                                   int T, int lm_pos_add, LaunchHook *hook) {
     cudaError_t e;
     int *err = b.ctrl + CTRL_ERR;
-    if ((e = launch_kernel(embed_rows_kernel, dim3(T), 256, 0, st, 1, true, b.W + p.w_embed, b.tok, b.X, p.H)) !=
+    if ((e = launch_kernel(embed_rows_kernel, dim3(T), 256, 0, st, 1, p.pdl, b.W + p.w_embed, b.tok, b.X, p.H)) !=
         cudaSuccess)
         return e;
     for (int l = 0; l < p.L; ++l) {
@@ -367,7 +367,7 @@ cudaError_t enqueue_prefill_chunk(const Plan &p, const Bufs &b, const PrefillMap
         uint16_t *kvl = b.KV + (size_t)l * p.kv_layer_elems;
         // A3 + A4: RMSNorm, QKV (+bias), RoPE, paged KV append
         const Terms A = {{b.A[0], b.A[1], b.A[2]}};
-        if ((e = launch_kernel(rmsnorm_rows_kernel, dim3(T), 256, 0, st, 1, true, b.X, b.W + lo.attn_norm, A, p.H,
+        if ((e = launch_kernel(rmsnorm_rows_kernel, dim3(T), 256, 0, st, 1, p.pdl, b.X, b.W + lo.attn_norm, A, p.H,
                                p.cfg.rms_eps, PEpiQKV::kATerms)) != cudaSuccess)
             return e;
         PEpiQKV eq = {{{b.Q[0], b.Q[1], b.Q[2]}}, kvl, b.pages, b.rope, p.cfg.qkv_bias ? b.W + lo.bqkv : nullptr, P, p.qdim,
@@ -383,7 +383,7 @@ cudaError_t enqueue_prefill_chunk(const Plan &p, const Bufs &b, const PrefillMap
             const Terms Qt = {{b.Q[0], b.Q[1], b.Q[2]}};
             const dim3 grid(T, (p.nq + p.nkv + 7) / 8);
             if (hook) hook->before("prefill_qk_norm_rope");
-            e = launch_kernel(p.d == 128 ? qk_norm_rope_kernel<128> : qk_norm_rope_kernel<64>, grid, 256, 0, st, 1, true,
+            e = launch_kernel(p.d == 128 ? qk_norm_rope_kernel<128> : qk_norm_rope_kernel<64>, grid, 256, 0, st, 1, p.pdl,
                               b.QKraw, b.W + lo.qn, b.W + lo.kn, b.rope, Qt, kvl, b.pages, p.kv_page_elems, P, p.nq,
                               p.nkv, p.cfg.rms_eps);
             if (hook) hook->after("prefill_qk_norm_rope");
@@ -402,7 +402,7 @@ cudaError_t enqueue_prefill_chunk(const Plan &p, const Bufs &b, const PrefillMap
                       "prefill_o_proj")) != cudaSuccess)
             return e;
         // A7: RMSNorm + gate/up + SwiGLU
-        if ((e = launch_kernel(rmsnorm_rows_kernel, dim3(T), 256, 0, st, 1, true, b.X, b.W + lo.ffn_norm, A, p.H,
+        if ((e = launch_kernel(rmsnorm_rows_kernel, dim3(T), 256, 0, st, 1, p.pdl, b.X, b.W + lo.ffn_norm, A, p.H,
                                p.cfg.rms_eps, PEpiSwiGLU::kATerms)) != cudaSuccess)
             return e;
         const Terms M = {{b.M[0], b.M[1], b.M[2]}};
@@ -422,7 +422,7 @@ cudaError_t enqueue_prefill_chunk(const Plan &p, const Bufs &b, const PrefillMap
     }
     if (lm_pos_add > 0) {
         // A9 on the chunk's last row only
-        return enqueue_lm_head(p, b, b.X + (size_t)(T - 1) * p.H, st, true, lm_pos_add, hook);
+        return enqueue_lm_head(p, b, b.X + (size_t)(T - 1) * p.H, st, p.pdl, lm_pos_add, hook);
     }
     return cudaSuccess;
 }

@@ -54,6 +54,10 @@ struct Plan {
     size_t wt_elems;        // elements of the largest per-layer matrix
     size_t ws_bytes;
     int num_sms;
+    // Programmatic dependent launch of the prefill's kernels.  A kernel that starts early takes
+    // SMs beside its predecessor's and holds them while it waits, so a context with an SM share
+    // launches without it.
+    bool pdl;
 };
 
 // Fills `p` from `cfg`; returns an error message or nullptr.

@@ -304,23 +304,23 @@ cudaError_t launch_gemm(const Plan &p, const GemmMaps &maps, int terms, int T, i
     const dim3 grid(SPLIT > 1 ? tiles * SPLIT : tiles < p.num_sms ? tiles : p.num_sms);
     constexpr size_t smem = TcTile<BN, STACK ? 1 : Epi::kATerms>::SMEM;
     if (terms == 1)
-        return launch_kernel(gemm_tc_kernel<BN, SPLIT, STACK, 1, Epi>, grid, TC_THREADS, smem, st, SPLIT, true, maps, T, N, K, err,
+        return launch_kernel(gemm_tc_kernel<BN, SPLIT, STACK, 1, Epi>, grid, TC_THREADS, smem, st, SPLIT, p.pdl, maps, T, N, K, err,
                              epi);
-    return launch_kernel(gemm_tc_kernel<BN, SPLIT, STACK, kTerms, Epi>, grid, TC_THREADS, smem, st, SPLIT, true, maps, T, N, K,
+    return launch_kernel(gemm_tc_kernel<BN, SPLIT, STACK, kTerms, Epi>, grid, TC_THREADS, smem, st, SPLIT, p.pdl, maps, T, N, K,
                          err, epi);
 }
 
 template <int BN, class Epi>
-cudaError_t launch_gemm_pair(int pairs, const GemmMaps &maps, int terms, int T, int N, int K, int *err,
+cudaError_t launch_gemm_pair(const Plan &p, int pairs, const GemmMaps &maps, int terms, int T, int N, int K, int *err,
                                     const Epi &epi, cudaStream_t st) {
     const int tiles = ((T + 2 * TC_BM - 1) / (2 * TC_BM)) * ((N + BN - 1) / BN);
     const int grid = 2 * (tiles < pairs ? tiles : pairs);
     constexpr size_t smem = TcPairTile<BN, Epi::kATerms>::SMEM;
     // __cluster_dims__ gives the pairs
     if (terms == 1)
-        return launch_kernel(gemm2_tc_kernel<BN, 1, Epi>, dim3(grid), TC_THREADS, smem, st, 1, true, maps, T, N, K, err,
+        return launch_kernel(gemm2_tc_kernel<BN, 1, Epi>, dim3(grid), TC_THREADS, smem, st, 1, p.pdl, maps, T, N, K, err,
                              epi);
-    return launch_kernel(gemm2_tc_kernel<BN, kTerms, Epi>, dim3(grid), TC_THREADS, smem, st, 1, true, maps, T, N, K, err,
+    return launch_kernel(gemm2_tc_kernel<BN, kTerms, Epi>, dim3(grid), TC_THREADS, smem, st, 1, p.pdl, maps, T, N, K, err,
                          epi);
 }
 
@@ -349,9 +349,9 @@ cudaError_t gemm(const Plan &p, const PrefillMaps &mp, const MatrixMaps (&a)[kTe
     };
     using std::integral_constant;
     if (c.pair)
-        e = c.bn == 256   ? launch_gemm_pair<256>(mp.pairs, maps, w.terms, T, N, K, err, epi, st)
-            : c.bn == 224 ? launch_gemm_pair<224>(mp.pairs, maps, w.terms, T, N, K, err, epi, st)
-                          : launch_gemm_pair<192>(mp.pairs, maps, w.terms, T, N, K, err, epi, st);
+        e = c.bn == 256   ? launch_gemm_pair<256>(p, mp.pairs, maps, w.terms, T, N, K, err, epi, st)
+            : c.bn == 224 ? launch_gemm_pair<224>(p, mp.pairs, maps, w.terms, T, N, K, err, epi, st)
+                          : launch_gemm_pair<192>(p, mp.pairs, maps, w.terms, T, N, K, err, epi, st);
     else if (c.bn == 128 && !c.stack)
         e = shared(integral_constant<int, 128>(), std::false_type());
     else if (c.bn == 192 && !c.stack)

@@ -99,6 +99,7 @@ const char *wici::make_plan(const wici_config *cfg, int num_sms, Plan *p) {
     P.max_chunk = c.max_chunk;
     P.num_sms = num_sms > 0 ? num_sms : 1;
     if (c.max_sms > 0 && c.max_sms < P.num_sms) P.num_sms = c.max_sms;   // this tenant's SM share
+    P.pdl = c.max_sms == 0;
     P.q8 = c.weight_format == WICI_WEIGHTS_Q8;
     P.qk_norm = c.qk_norm == 1;
 
