@@ -5,10 +5,9 @@
 #include <stdarg.h>
 #include <stdio.h>
 
-#include <mutex>
-
 #include "../../include/wici.h"
 #include "conv2_tc.cuh"
+#include "conv_plan.h"
 #include "conv_tc.cuh"
 #include "kernels.h"
 
@@ -38,9 +37,7 @@ const char *check_shape(const wici_conv_shape *s) {
 
 bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
-std::mutex g_mu;
-int g_attr_device = -1;
-int g_sms = 0, g_clusters[4] = {};   // SMs; resident clusters of 1, 2, 4 and 8 CTAs
+ConvDevices g_devices;
 
 template <int MODE>
 cudaError_t setup_mode() {
@@ -69,24 +66,23 @@ cudaError_t count_clusters(int nsm, int *n) {
     return cudaOccupancyMaxActiveClusters(n, conv_tc_kernel<CONV_FWD, SPLIT>, &cfg);
 }
 
-// once per device (the last one used is remembered)
-cudaError_t setup() {
+// the current device's counts, with the kernels' shared-memory limits set there
+cudaError_t setup(ConvDevice *out) {
     int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    std::lock_guard<std::mutex> lk(g_mu);
-    if (g_attr_device == dev) return cudaSuccess;
-    if ((e = cudaDeviceGetAttribute(&g_sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
-        (e = setup_mode<CONV_FWD>()) != cudaSuccess || (e = setup_mode<CONV_DGRAD>()) != cudaSuccess ||
-        (e = setup_mode<CONV_WGRAD>()) != cudaSuccess)
-        return e;
-    g_clusters[0] = g_sms;
-    if ((e = count_clusters<2>(g_sms, &g_clusters[1])) != cudaSuccess ||
-        (e = count_clusters<4>(g_sms, &g_clusters[2])) != cudaSuccess ||
-        (e = count_clusters<8>(g_sms, &g_clusters[3])) != cudaSuccess)
-        return e;
-    g_attr_device = dev;
-    return cudaSuccess;
+    if (const cudaError_t e = cudaGetDevice(&dev)) return e;
+    return g_devices.get(dev, out, [dev](ConvDevice *d) {
+        cudaError_t e;
+        if ((e = cudaDeviceGetAttribute(&d->sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+            (e = setup_mode<CONV_FWD>()) != cudaSuccess || (e = setup_mode<CONV_DGRAD>()) != cudaSuccess ||
+            (e = setup_mode<CONV_WGRAD>()) != cudaSuccess)
+            return e;
+        d->clusters[0] = d->sms;
+        if ((e = count_clusters<2>(d->sms, &d->clusters[1])) != cudaSuccess ||
+            (e = count_clusters<4>(d->sms, &d->clusters[2])) != cudaSuccess ||
+            (e = count_clusters<8>(d->sms, &d->clusters[3])) != cudaSuccess)
+            return e;
+        return cudaSuccess;
+    });
 }
 
 ConvArgs make_args(const wici_conv_shape *s, float *out, void *ws) {
@@ -134,16 +130,16 @@ bool map_rows(CUtensorMap *m, const void *ptr, uint64_t rows, uint64_t cols, int
 // SM cycles: waves of tiles x (blocks of a CTA x 512 cycles of MMAs + the pipeline's fill
 // and the epilogue, and the exchange of a split tile).  A single CTA takes about 640
 // cycles a block (its ports serve all of B), a pair 540.
-int pick_ctas(int tiles, int pair_tiles, int nkb) {
+int pick_ctas(const ConvDevice &d, int tiles, int pair_tiles, int nkb) {
     auto cost = [](int units, int slots, double blocks, double cycles, double fixed) {
         return (double)((units + slots - 1) / slots) * (blocks * cycles + fixed);
     };
     int best = 0;
-    double best_cost = cost(pair_tiles, g_clusters[1], nkb, 540.0, 5000.0);
+    double best_cost = cost(pair_tiles, d.clusters[1], nkb, 540.0, 5000.0);
     for (int i = 0; i < 4; ++i) {
-        if (g_clusters[i] == 0) continue;
+        if (d.clusters[i] == 0) continue;
         const int split = 1 << i;
-        const double c = cost(tiles, g_clusters[i], (nkb + split - 1) / split, 640.0, i == 0 ? 4000.0 : 7000.0);
+        const double c = cost(tiles, d.clusters[i], (nkb + split - 1) / split, 640.0, i == 0 ? 4000.0 : 7000.0);
         if (c < best_cost) {
             best = split;
             best_cost = c;
@@ -153,26 +149,28 @@ int pick_ctas(int tiles, int pair_tiles, int nkb) {
 }
 
 template <int MODE, int SPLIT>
-cudaError_t launch_split(const CUtensorMap &ma, const CUtensorMap &mb, const ConvArgs &a, cudaStream_t st) {
+cudaError_t launch_split(const ConvDevice &d, const CUtensorMap &ma, const CUtensorMap &mb, const ConvArgs &a,
+                         cudaStream_t st) {
     // one tile per cluster where tiles are shared, otherwise persistent
-    const int grid = SPLIT > 1 ? a.ntiles * SPLIT : a.ntiles < g_sms ? a.ntiles : g_sms;
+    const int grid = SPLIT > 1 ? a.ntiles * SPLIT : a.ntiles < d.sms ? a.ntiles : d.sms;
     return launch_kernel(conv_tc_kernel<MODE, SPLIT>, dim3(grid), CV_THREADS, CV_SMEM, st, SPLIT, true, ma, mb, a);
 }
 
 // ctas: pick_ctas; mb: boxes of 128 rows for pairs, of 256 otherwise (the same for the filter gradient)
 template <int MODE>
-cudaError_t launch(int ctas, const CUtensorMap &ma, const CUtensorMap &mb, ConvArgs a, int tiles, cudaStream_t st) {
+cudaError_t launch(const ConvDevice &d, int ctas, const CUtensorMap &ma, const CUtensorMap &mb, ConvArgs a, int tiles,
+                   cudaStream_t st) {
     a.ntiles = ctas == 0 ? cv_pair_tiles<MODE>(a) : tiles;
     switch (ctas) {
         case 0: {
-            const int grid = 2 * (a.ntiles < g_clusters[1] ? a.ntiles : g_clusters[1]);
+            const int grid = 2 * (a.ntiles < d.clusters[1] ? a.ntiles : d.clusters[1]);
             // __cluster_dims__ gives the pairs
             return launch_kernel(conv2_tc_kernel<MODE>, dim3(grid), CV_THREADS, CV2_SMEM, st, 1, true, ma, mb, a);
         }
-        case 1: return launch_split<MODE, 1>(ma, mb, a, st);
-        case 2: return launch_split<MODE, 2>(ma, mb, a, st);
-        case 4: return launch_split<MODE, 4>(ma, mb, a, st);
-        default: return launch_split<MODE, 8>(ma, mb, a, st);
+        case 1: return launch_split<MODE, 1>(d, ma, mb, a, st);
+        case 2: return launch_split<MODE, 2>(d, ma, mb, a, st);
+        case 4: return launch_split<MODE, 4>(d, ma, mb, a, st);
+        default: return launch_split<MODE, 8>(d, ma, mb, a, st);
     }
 }
 
@@ -192,16 +190,17 @@ int wici_conv_forward(void *cuda_stream, const wici_conv_shape *s, const void *x
     if (const char *m = check_shape(s)) return fail(WICI_E_ARG, "conv: %s", m);
     if (!aligned16(x) || !aligned16(w) || !aligned16(y) || !aligned16(workspace) || !workspace)
         return fail(WICI_E_ARG, "conv: null or unaligned buffer");
-    cudaError_t e = setup();
+    ConvDevice dev;
+    cudaError_t e = setup(&dev);
     if (e != cudaSuccess) return fail(WICI_E_CUDA, "conv: %s", cudaGetErrorString(e));
     CUtensorMap ma, mb;
     const ConvArgs a = make_args(s, y, workspace);
     const int tiles = a.n * a.pt * a.qt * (a.k / CV_BN);
-    const int ctas = pick_ctas(tiles, cv_pair_tiles<CONV_FWD>(a), 9 * (a.c / CV_BK));
+    const int ctas = pick_ctas(dev, tiles, cv_pair_tiles<CONV_FWD>(a), 9 * (a.c / CV_BK));
     if (!map_x_strided(&ma, x, s, 32, 16) ||
         !map_rows(&mb, w, (uint64_t)s->k, (uint64_t)9 * s->c, ctas == 0 ? CV_BN / 2 : CV_BN))
         return fail(WICI_E_CUDA, "conv: cuTensorMapEncodeTiled failed");
-    if ((e = launch<CONV_FWD>(ctas, ma, mb, a, tiles, (cudaStream_t)cuda_stream)) != cudaSuccess)
+    if ((e = launch<CONV_FWD>(dev, ctas, ma, mb, a, tiles, (cudaStream_t)cuda_stream)) != cudaSuccess)
         return fail(WICI_E_CUDA, "conv forward: %s", cudaGetErrorString(e));
     return WICI_OK;
 }
@@ -211,7 +210,8 @@ int wici_conv_backward_data(void *cuda_stream, const wici_conv_shape *s, const v
     if (const char *m = check_shape(s)) return fail(WICI_E_ARG, "conv: %s", m);
     if (!aligned16(dy) || !aligned16(w) || !aligned16(dx) || !aligned16(workspace) || !workspace)
         return fail(WICI_E_ARG, "conv: null or unaligned buffer");
-    cudaError_t e = setup();
+    ConvDevice dev;
+    cudaError_t e = setup(&dev);
     if (e != cudaSuccess) return fail(WICI_E_CUDA, "conv: %s", cudaGetErrorString(e));
     cudaStream_t st = (cudaStream_t)cuda_stream;
     uint16_t *wt = (uint16_t *)((uint8_t *)workspace + kConvErrBytes);
@@ -221,11 +221,11 @@ int wici_conv_backward_data(void *cuda_stream, const wici_conv_shape *s, const v
     CUtensorMap ma, mb;
     const ConvArgs a = make_args(s, dx, workspace);
     const int tiles = 4 * a.n * a.pt * a.qt * (a.c / CV_BN);
-    const int ctas = pick_ctas(tiles, cv_pair_tiles<CONV_DGRAD>(a), 4 * (a.k / CV_BK));
+    const int ctas = pick_ctas(dev, tiles, cv_pair_tiles<CONV_DGRAD>(a), 4 * (a.k / CV_BK));
     if (!map_dy(&ma, dy, s, 8) ||
         !map_rows(&mb, wt, (uint64_t)9 * s->c, (uint64_t)s->k, ctas == 0 ? CV_BN / 2 : CV_BN))
         return fail(WICI_E_CUDA, "conv: cuTensorMapEncodeTiled failed");
-    if ((e = launch<CONV_DGRAD>(ctas, ma, mb, a, tiles, st)) != cudaSuccess)
+    if ((e = launch<CONV_DGRAD>(dev, ctas, ma, mb, a, tiles, st)) != cudaSuccess)
         return fail(WICI_E_CUDA, "conv data gradient: %s", cudaGetErrorString(e));
     return WICI_OK;
 }
@@ -235,15 +235,16 @@ int wici_conv_backward_filter(void *cuda_stream, const wici_conv_shape *s, const
     if (const char *m = check_shape(s)) return fail(WICI_E_ARG, "conv: %s", m);
     if (!aligned16(x) || !aligned16(dy) || !aligned16(dw) || !aligned16(workspace) || !workspace)
         return fail(WICI_E_ARG, "conv: null or unaligned buffer");
-    cudaError_t e = setup();
+    ConvDevice dev;
+    cudaError_t e = setup(&dev);
     if (e != cudaSuccess) return fail(WICI_E_CUDA, "conv: %s", cudaGetErrorString(e));
     CUtensorMap ma, mb;
     if (!map_dy(&ma, dy, s, 4) || !map_x_strided(&mb, x, s, 32, 8))
         return fail(WICI_E_CUDA, "conv: cuTensorMapEncodeTiled failed");
     const ConvArgs a = make_args(s, dw, workspace);
     const int tiles = 9 * (a.k / CV_BM) * (a.c / CV_BN);
-    const int ctas = pick_ctas(tiles, cv_pair_tiles<CONV_WGRAD>(a), a.n * ((a.p + 3) / 4) * a.qt);
-    if ((e = launch<CONV_WGRAD>(ctas, ma, mb, a, tiles, (cudaStream_t)cuda_stream)) != cudaSuccess)
+    const int ctas = pick_ctas(dev, tiles, cv_pair_tiles<CONV_WGRAD>(a), a.n * ((a.p + 3) / 4) * a.qt);
+    if ((e = launch<CONV_WGRAD>(dev, ctas, ma, mb, a, tiles, (cudaStream_t)cuda_stream)) != cudaSuccess)
         return fail(WICI_E_CUDA, "conv filter gradient: %s", cudaGetErrorString(e));
     return WICI_OK;
 }
