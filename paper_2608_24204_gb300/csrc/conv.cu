@@ -125,29 +125,6 @@ bool map_rows(CUtensorMap *m, const void *ptr, uint64_t rows, uint64_t cols, int
     return encode_tiled(m, 2, ptr, dims, st, box, es);
 }
 
-// How a layer's `tiles` of 128 x 256 outputs with `nkb` reduction blocks (the longest tile's)
-// run: on pairs of CTAs (0), one CTA a tile (1), or 2, 4 or 8 CTAs sharing one.  Modelled
-// SM cycles: waves of tiles x (blocks of a CTA x 512 cycles of MMAs + the pipeline's fill
-// and the epilogue, and the exchange of a split tile).  A single CTA takes about 640
-// cycles a block (its ports serve all of B), a pair 540.
-int pick_ctas(const ConvDevice &d, int tiles, int pair_tiles, int nkb) {
-    auto cost = [](int units, int slots, double blocks, double cycles, double fixed) {
-        return (double)((units + slots - 1) / slots) * (blocks * cycles + fixed);
-    };
-    int best = 0;
-    double best_cost = cost(pair_tiles, d.clusters[1], nkb, 540.0, 5000.0);
-    for (int i = 0; i < 4; ++i) {
-        if (d.clusters[i] == 0) continue;
-        const int split = 1 << i;
-        const double c = cost(tiles, d.clusters[i], (nkb + split - 1) / split, 640.0, i == 0 ? 4000.0 : 7000.0);
-        if (c < best_cost) {
-            best = split;
-            best_cost = c;
-        }
-    }
-    return best;
-}
-
 template <int MODE, int SPLIT>
 cudaError_t launch_split(const ConvDevice &d, const CUtensorMap &ma, const CUtensorMap &mb, const ConvArgs &a,
                          cudaStream_t st) {

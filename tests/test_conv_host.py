@@ -55,3 +55,24 @@ def test_each_device_keeps_its_own_counts(tmp_path):
     CHECK(wrong[0] == 0 && wrong[1] == 0);
     CHECK(asked[0] == 1 && asked[1] == 1);
     """)
+
+
+def test_ctas_per_tile_on_devices_without_some_cluster_sizes(tmp_path):
+    # no resident pair (a small or partitioned device): one CTA per tile is always there; where
+    # pairs and clusters exist, large layers take pairs and small ones clusters
+    run_host(tmp_path, r"""
+    ConvDevice none, solo, all;
+    none.sms = solo.sms = all.sms = 152;
+    solo.clusters[0] = 1;
+    const int n[4] = {152, 76, 36, 16};
+    for (int i = 0; i < 4; ++i) all.clusters[i] = n[i];
+    for (int tiles : {1, 2, 3, 9, 64, 1000, 50000})
+        for (int nkb : {1, 4, 36, 144, 800}) {
+            CHECK(pick_ctas(none, tiles, (tiles + 1) / 2, nkb) == 1);
+            CHECK(pick_ctas(solo, tiles, (tiles + 1) / 2, nkb) == 1);
+            const int c = pick_ctas(all, tiles, (tiles + 1) / 2, nkb);
+            CHECK(c == 0 || c == 1 || c == 2 || c == 4 || c == 8);
+        }
+    CHECK(pick_ctas(all, 1568, 784, 144) == 0);
+    CHECK(pick_ctas(all, 2, 1, 144) == 8);
+    """)
