@@ -33,7 +33,6 @@ namespace wici {
 // us with five grid barriers a layer, 70 us now; at 1B widths 35.0 and 27.5 us.
 constexpr int kMegaSlots = 6;
 constexpr uint32_t kMegaSlotBytes = 32768;
-constexpr int kMegaMaxCtas = 256;               // grid size limit (one CTA per SM)
 constexpr int kMaxSplits = 32;                  // attention splits of one KV head
 // attention scratch: per page set, per query head of the group, an O row, m and l
 constexpr size_t kMegaStateBytes = 21504;
@@ -1101,7 +1100,7 @@ __device__ bool mc_attn(MegaRing &R, const MegaArgs &a, uint16_t *kvl, const Meg
 // an even share.  Which CTA streams which rows changes no result.
 __device__ inline void mega_rebalance(const MegaArgs &a, float *scr) {
     const int G = gridDim.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    static_assert(kMegaMaxCtas <= kGemvConsumers, "one thread per CTA");
+    static_assert(kMaxCtas <= kGemvConsumers, "one thread per CTA");
     // sum of v over the consumers, with the inclusive prefix sums in *pre
     auto block_sum = [&](float v, float *pre) {
         float p = v;

@@ -163,7 +163,7 @@ static bool q8_shape_is(int K) {
 
 // the instantiation of this plan's widths and format, or nullptr
 static MegaLaunch mega_named_launcher(const Plan &p) {
-    if (p.qdim != p.H || p.num_sms > kMegaMaxCtas) return nullptr;
+    if (p.qdim != p.H) return nullptr;
 #define WICI_MEGA_PICK(DD, SH, SF, Q8, QH, QF)                                                       \
     if (p.q8 == Q8 && p.d == DD && shape_is<SH>(p.H) && shape_is<SF>(p.F) &&                            \
         (!Q8 || (q8_shape_is<QH>(p.H) && q8_shape_is<QF>(p.F))))                                        \
@@ -202,7 +202,7 @@ static cudaError_t enqueue_mega(const Plan &p, const Bufs &b, const CUtensorMap 
     // warps that take pages: as many as the group's states leave room for
     const int fit = (int)(kMegaStateBytes / ((size_t)p.group * (p.d + 4) * sizeof(float)));
     a.nsets = fit < kGemvWarps ? fit : kGemvWarps;
-    const int grid = p.num_sms < kMegaMaxCtas ? p.num_sms : kMegaMaxCtas;
+    const int grid = p.num_sms;   // the row-share table has an entry for each
     // one CTA per (KV head, split); more KV heads than CTAs: one split each
     a.splits = grid / p.nkv < 1 ? 1 : grid / p.nkv < kMaxSplits ? grid / p.nkv : kMaxSplits;
     a.bias = p.cfg.qkv_bias;

@@ -11,6 +11,7 @@
 namespace wici {
 
 constexpr int kPage = 16;          // tokens per KV page
+constexpr int kMaxCtas = 256;      // SMs a context uses at most: one row share per consumer thread of the decode step
 constexpr int kGemvThreads = 288;  // 8 consumer warps + 1 producer warp
 #ifndef WICI_GEMV_RING_BYTES
 #define WICI_GEMV_RING_BYTES 98304
@@ -53,7 +54,7 @@ struct Plan {
     size_t ws_QKraw;        // qk_norm only: the chunk's q|k before their norms (prefill)
     size_t wt_elems;        // elements of the largest per-layer matrix
     size_t ws_bytes;
-    int num_sms;
+    int num_sms;            // at most kMaxCtas: the decode step's grid and its table of row shares
     // Programmatic dependent launch of the prefill's kernels.  A kernel that starts early takes
     // SMs beside its predecessor's and holds them while it waits, so a context with an SM share
     // launches without it.

@@ -97,7 +97,7 @@ const char *wici::make_plan(const wici_config *cfg, int num_sms, Plan *p) {
     P.group = P.nq / P.nkv;
     P.max_pages = (c.max_tokens + kPage - 1) / kPage;
     P.max_chunk = c.max_chunk;
-    P.num_sms = num_sms > 0 ? num_sms : 1;
+    P.num_sms = num_sms < 1 ? 1 : num_sms < kMaxCtas ? num_sms : kMaxCtas;
     if (c.max_sms > 0 && c.max_sms < P.num_sms) P.num_sms = c.max_sms;   // this tenant's SM share
     P.pdl = c.max_sms == 0;
     P.q8 = c.weight_format == WICI_WEIGHTS_Q8;
