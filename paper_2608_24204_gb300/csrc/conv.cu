@@ -151,6 +151,86 @@ cudaError_t launch(const ConvDevice &d, int ctas, const CUtensorMap &ma, const C
     }
 }
 
+constexpr int kPick = -1;   // CTAs per tile: pick_ctas of the call's shape
+
+// the CTAs per tile of a call, or a negative number when the device has none resident that way
+int ctas_of(const ConvDevice &d, int ctas, int tiles, int pair_tiles, int nkb) {
+    if (ctas == kPick) return pick_ctas(d, tiles, pair_tiles, nkb);
+    switch (ctas) {
+        case 0: case 2: return d.clusters[1] > 0 ? ctas : kPick;
+        case 1: return ctas;
+        case 4: return d.clusters[2] > 0 ? ctas : kPick;
+        case 8: return d.clusters[3] > 0 ? ctas : kPick;
+        default: return kPick;
+    }
+}
+
+int forward(cudaStream_t st, const wici_conv_shape *s, const void *x, const void *w, float *y, void *workspace,
+            int ctas) {
+    if (const char *m = check_shape(s)) return fail(WICI_E_ARG, "conv: %s", m);
+    if (!aligned16(x) || !aligned16(w) || !aligned16(y) || !aligned16(workspace) || !workspace)
+        return fail(WICI_E_ARG, "conv: null or unaligned buffer");
+    ConvDevice dev;
+    cudaError_t e = setup(&dev);
+    if (e != cudaSuccess) return fail(WICI_E_CUDA, "conv: %s", cudaGetErrorString(e));
+    CUtensorMap ma, mb;
+    const ConvArgs a = make_args(s, y, workspace);
+    const int tiles = a.n * a.pt * a.qt * (a.k / CV_BN);
+    ctas = ctas_of(dev, ctas, tiles, cv_pair_tiles<CONV_FWD>(a), 9 * (a.c / CV_BK));
+    if (ctas < 0) return fail(WICI_E_ARG, "conv: CTAs per tile");
+    if (!map_x_strided(&ma, x, s, 32, 16) ||
+        !map_rows(&mb, w, (uint64_t)s->k, (uint64_t)9 * s->c, ctas == 0 ? CV_BN / 2 : CV_BN))
+        return fail(WICI_E_CUDA, "conv: cuTensorMapEncodeTiled failed");
+    if ((e = launch<CONV_FWD>(dev, ctas, ma, mb, a, tiles, st)) != cudaSuccess)
+        return fail(WICI_E_CUDA, "conv forward: %s", cudaGetErrorString(e));
+    return WICI_OK;
+}
+
+int backward_data(cudaStream_t st, const wici_conv_shape *s, const void *dy, const void *w, float *dx, void *workspace,
+                  int ctas) {
+    if (const char *m = check_shape(s)) return fail(WICI_E_ARG, "conv: %s", m);
+    if (!aligned16(dy) || !aligned16(w) || !aligned16(dx) || !aligned16(workspace) || !workspace)
+        return fail(WICI_E_ARG, "conv: null or unaligned buffer");
+    ConvDevice dev;
+    cudaError_t e = setup(&dev);
+    if (e != cudaSuccess) return fail(WICI_E_CUDA, "conv: %s", cudaGetErrorString(e));
+    const ConvArgs a = make_args(s, dx, workspace);
+    const int tiles = 4 * a.n * a.pt * a.qt * (a.c / CV_BN);
+    ctas = ctas_of(dev, ctas, tiles, cv_pair_tiles<CONV_DGRAD>(a), 4 * (a.k / CV_BK));
+    if (ctas < 0) return fail(WICI_E_ARG, "conv: CTAs per tile");
+    uint16_t *wt = (uint16_t *)((uint8_t *)workspace + kConvErrBytes);
+    if ((e = launch_kernel(conv_transpose_filter_kernel, dim3((s->c + 31) / 32, (s->k + 31) / 32, 9), 256, 0, st, 1,
+                           true, (const uint16_t *)w, wt, s->k, s->c)) != cudaSuccess)
+        return fail(WICI_E_CUDA, "conv transpose: %s", cudaGetErrorString(e));
+    CUtensorMap ma, mb;
+    if (!map_dy(&ma, dy, s, 8) ||
+        !map_rows(&mb, wt, (uint64_t)9 * s->c, (uint64_t)s->k, ctas == 0 ? CV_BN / 2 : CV_BN))
+        return fail(WICI_E_CUDA, "conv: cuTensorMapEncodeTiled failed");
+    if ((e = launch<CONV_DGRAD>(dev, ctas, ma, mb, a, tiles, st)) != cudaSuccess)
+        return fail(WICI_E_CUDA, "conv data gradient: %s", cudaGetErrorString(e));
+    return WICI_OK;
+}
+
+int backward_filter(cudaStream_t st, const wici_conv_shape *s, const void *x, const void *dy, float *dw,
+                    void *workspace, int ctas) {
+    if (const char *m = check_shape(s)) return fail(WICI_E_ARG, "conv: %s", m);
+    if (!aligned16(x) || !aligned16(dy) || !aligned16(dw) || !aligned16(workspace) || !workspace)
+        return fail(WICI_E_ARG, "conv: null or unaligned buffer");
+    ConvDevice dev;
+    cudaError_t e = setup(&dev);
+    if (e != cudaSuccess) return fail(WICI_E_CUDA, "conv: %s", cudaGetErrorString(e));
+    CUtensorMap ma, mb;
+    if (!map_dy(&ma, dy, s, 4) || !map_x_strided(&mb, x, s, 32, 8))
+        return fail(WICI_E_CUDA, "conv: cuTensorMapEncodeTiled failed");
+    const ConvArgs a = make_args(s, dw, workspace);
+    const int tiles = 9 * (a.k / CV_BM) * (a.c / CV_BN);
+    ctas = ctas_of(dev, ctas, tiles, cv_pair_tiles<CONV_WGRAD>(a), a.n * ((a.p + 3) / 4) * a.qt);
+    if (ctas < 0) return fail(WICI_E_ARG, "conv: CTAs per tile");
+    if ((e = launch<CONV_WGRAD>(dev, ctas, ma, mb, a, tiles, st)) != cudaSuccess)
+        return fail(WICI_E_CUDA, "conv filter gradient: %s", cudaGetErrorString(e));
+    return WICI_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -164,66 +244,29 @@ int wici_conv_workspace_bytes(const wici_conv_shape *s, size_t *bytes) {
 
 int wici_conv_forward(void *cuda_stream, const wici_conv_shape *s, const void *x, const void *w, float *y,
                       void *workspace) {
-    if (const char *m = check_shape(s)) return fail(WICI_E_ARG, "conv: %s", m);
-    if (!aligned16(x) || !aligned16(w) || !aligned16(y) || !aligned16(workspace) || !workspace)
-        return fail(WICI_E_ARG, "conv: null or unaligned buffer");
-    ConvDevice dev;
-    cudaError_t e = setup(&dev);
-    if (e != cudaSuccess) return fail(WICI_E_CUDA, "conv: %s", cudaGetErrorString(e));
-    CUtensorMap ma, mb;
-    const ConvArgs a = make_args(s, y, workspace);
-    const int tiles = a.n * a.pt * a.qt * (a.k / CV_BN);
-    const int ctas = pick_ctas(dev, tiles, cv_pair_tiles<CONV_FWD>(a), 9 * (a.c / CV_BK));
-    if (!map_x_strided(&ma, x, s, 32, 16) ||
-        !map_rows(&mb, w, (uint64_t)s->k, (uint64_t)9 * s->c, ctas == 0 ? CV_BN / 2 : CV_BN))
-        return fail(WICI_E_CUDA, "conv: cuTensorMapEncodeTiled failed");
-    if ((e = launch<CONV_FWD>(dev, ctas, ma, mb, a, tiles, (cudaStream_t)cuda_stream)) != cudaSuccess)
-        return fail(WICI_E_CUDA, "conv forward: %s", cudaGetErrorString(e));
-    return WICI_OK;
+    return forward((cudaStream_t)cuda_stream, s, x, w, y, workspace, kPick);
 }
 
 int wici_conv_backward_data(void *cuda_stream, const wici_conv_shape *s, const void *dy, const void *w, float *dx,
                             void *workspace) {
-    if (const char *m = check_shape(s)) return fail(WICI_E_ARG, "conv: %s", m);
-    if (!aligned16(dy) || !aligned16(w) || !aligned16(dx) || !aligned16(workspace) || !workspace)
-        return fail(WICI_E_ARG, "conv: null or unaligned buffer");
-    ConvDevice dev;
-    cudaError_t e = setup(&dev);
-    if (e != cudaSuccess) return fail(WICI_E_CUDA, "conv: %s", cudaGetErrorString(e));
-    cudaStream_t st = (cudaStream_t)cuda_stream;
-    uint16_t *wt = (uint16_t *)((uint8_t *)workspace + kConvErrBytes);
-    if ((e = launch_kernel(conv_transpose_filter_kernel, dim3((s->c + 31) / 32, (s->k + 31) / 32, 9), 256, 0, st, 1, true,
-                           (const uint16_t *)w, wt, s->k, s->c)) != cudaSuccess)
-        return fail(WICI_E_CUDA, "conv transpose: %s", cudaGetErrorString(e));
-    CUtensorMap ma, mb;
-    const ConvArgs a = make_args(s, dx, workspace);
-    const int tiles = 4 * a.n * a.pt * a.qt * (a.c / CV_BN);
-    const int ctas = pick_ctas(dev, tiles, cv_pair_tiles<CONV_DGRAD>(a), 4 * (a.k / CV_BK));
-    if (!map_dy(&ma, dy, s, 8) ||
-        !map_rows(&mb, wt, (uint64_t)9 * s->c, (uint64_t)s->k, ctas == 0 ? CV_BN / 2 : CV_BN))
-        return fail(WICI_E_CUDA, "conv: cuTensorMapEncodeTiled failed");
-    if ((e = launch<CONV_DGRAD>(dev, ctas, ma, mb, a, tiles, st)) != cudaSuccess)
-        return fail(WICI_E_CUDA, "conv data gradient: %s", cudaGetErrorString(e));
-    return WICI_OK;
+    return backward_data((cudaStream_t)cuda_stream, s, dy, w, dx, workspace, kPick);
 }
 
 int wici_conv_backward_filter(void *cuda_stream, const wici_conv_shape *s, const void *x, const void *dy, float *dw,
                               void *workspace) {
-    if (const char *m = check_shape(s)) return fail(WICI_E_ARG, "conv: %s", m);
-    if (!aligned16(x) || !aligned16(dy) || !aligned16(dw) || !aligned16(workspace) || !workspace)
-        return fail(WICI_E_ARG, "conv: null or unaligned buffer");
-    ConvDevice dev;
-    cudaError_t e = setup(&dev);
-    if (e != cudaSuccess) return fail(WICI_E_CUDA, "conv: %s", cudaGetErrorString(e));
-    CUtensorMap ma, mb;
-    if (!map_dy(&ma, dy, s, 4) || !map_x_strided(&mb, x, s, 32, 8))
-        return fail(WICI_E_CUDA, "conv: cuTensorMapEncodeTiled failed");
-    const ConvArgs a = make_args(s, dw, workspace);
-    const int tiles = 9 * (a.k / CV_BM) * (a.c / CV_BN);
-    const int ctas = pick_ctas(dev, tiles, cv_pair_tiles<CONV_WGRAD>(a), a.n * ((a.p + 3) / 4) * a.qt);
-    if ((e = launch<CONV_WGRAD>(dev, ctas, ma, mb, a, tiles, (cudaStream_t)cuda_stream)) != cudaSuccess)
-        return fail(WICI_E_CUDA, "conv filter gradient: %s", cudaGetErrorString(e));
-    return WICI_OK;
+    return backward_filter((cudaStream_t)cuda_stream, s, x, dy, dw, workspace, kPick);
+}
+
+int wici_internal_conv(int mode, int ctas, void *cuda_stream, const wici_conv_shape *s, const void *a, const void *b,
+                       float *out, void *workspace) {
+    if (ctas == kPick) return fail(WICI_E_ARG, "conv: CTAs per tile");
+    cudaStream_t st = (cudaStream_t)cuda_stream;
+    switch (mode) {
+        case CONV_FWD: return forward(st, s, a, b, out, workspace, ctas);
+        case CONV_DGRAD: return backward_data(st, s, a, b, out, workspace, ctas);
+        case CONV_WGRAD: return backward_filter(st, s, a, b, out, workspace, ctas);
+        default: return fail(WICI_E_ARG, "conv: mode");
+    }
 }
 
 int wici_conv_status(void *cuda_stream, void *workspace) {

@@ -117,6 +117,12 @@ void set_thread_error(const char *msg);
 // RoPE table for positions [0, max_tokens).
 cudaError_t enqueue_rope_table(const Plan &p, const Bufs &b, cudaStream_t st);
 
+// Not part of the C ABI (tests): one pass of the convolution layer, mode 0 forward (a = x, b = w),
+// 1 data gradient (dy, w), 2 filter gradient (x, dy), with the CTAs per tile given (0: a pair on a
+// tile of 256 rows; 1, 2, 4 or 8) instead of picked.  WICI_E_ARG where the device has no such cluster.
+extern "C" int wici_internal_conv(int mode, int ctas, void *cuda_stream, const wici_conv_shape *s, const void *a,
+                                  const void *b, float *out, void *workspace);
+
 // One CTA waiting on an mbarrier that never completes; writes the wait's
 // site id to *err when it gives up after limit_ns.
 cudaError_t enqueue_bounded_wait_probe(int *err, int64_t limit_ns, cudaStream_t st);
