@@ -9,6 +9,7 @@
 #include "conv2_tc.cuh"
 #include "conv_plan.h"
 #include "conv_tc.cuh"
+#include "device_table.h"
 #include "kernels.h"
 
 using namespace wici;
@@ -37,7 +38,7 @@ const char *check_shape(const wici_conv_shape *s) {
 
 bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
-ConvDevices g_devices;
+DeviceTable<ConvDevice> g_devices;
 
 template <int MODE>
 cudaError_t setup_mode() {

@@ -745,7 +745,7 @@ __device__ __forceinline__ bool mc_phase(MegaRing &R, float *red, int K, int n_u
 // q and P are fp32 values split into three bf16 terms (24 bits: their fp32
 // precision) and K and V are exact bf16, so every product is exact.  The sums are fp32
 // in the accumulators, O's over every page that a warp takes: its error against 64 bits
-// grows with them (8B widths, 8000 keys: 3.2e-7 at one or two pages a warp, 7.0e-7 at 63)
+// grows with them (8B widths, 8000 keys: 3.2e-7 at four pages a warp, 7.0e-7 at 63)
 // and stays below that of fp32 FMAs in its place (8.5e-7).  A scalar version (one warp per head and page, lane-transposed dot
 // products) took about 1 us per page: 29 us a layer at 8K cached tokens.
 // The warps' states (O, m, l) are merged in shared memory and published as tagged

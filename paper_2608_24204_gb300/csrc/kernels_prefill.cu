@@ -9,11 +9,11 @@
 #include <math.h>
 #include <stdint.h>
 
-#include <mutex>
 #include <type_traits>
 
 #include "common.cuh"
 #include "attn_tc.cuh"
+#include "device_table.h"
 #include "kernels.h"
 #include "prefill_gemm.cuh"
 
@@ -290,32 +290,31 @@ const char *make_prefill_maps(const Plan &p, const Bufs &b, PrefillMaps *m) {
         m->wd.push_back(matrix(b.W + lo.wd, p.H, p.F));
     }
     m->sms = p.num_sms;
-    // kernel limits and resident clusters: once per device
-    static std::mutex mu;
-    static int dev_pairs[64] = {}, dev_quads[64] = {};
+    // kernel limits and resident clusters (there may be none): once per device
+    struct Clusters {
+        int pairs = 0, quads = 0;
+    };
+    static DeviceTable<Clusters> devices;
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return "no CUDA device";
-    {
-        std::lock_guard<std::mutex> lk(mu);
-        if (dev_pairs[dev] == 0) {
-            const auto limit = [](const void *f, size_t bytes) {
-                return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
-            };
-            int pairs = 0, quads = 0;
-            if (setup_gemm<PEpiQKV>() != cudaSuccess || setup_gemm<PEpiResidual>() != cudaSuccess ||
-                setup_gemm<PEpiSwiGLU>() != cudaSuccess ||
-                !limit((const void *)attn_tc_kernel<128>, AttnSmem<128>::TOTAL + 1024) ||
-                !limit((const void *)attn_tc_kernel<64>, AttnSmem<64>::TOTAL + 1024))
-                return "cannot raise the shared-memory limits of the prefill kernels";
-            if (resident_clusters<PEpiSwiGLU>(2, &pairs) != cudaSuccess ||
-                resident_clusters<PEpiSwiGLU>(4, &quads) != cudaSuccess || pairs < 1)
-                return "cannot query the resident clusters of the tensor-core GEMM";
-            dev_pairs[dev] = pairs;
-            dev_quads[dev] = quads;
-        }
-        m->pairs = dev_pairs[dev] < p.num_sms / 2 ? dev_pairs[dev] : p.num_sms / 2;
-        m->quads = dev_quads[dev] < p.num_sms / 4 ? dev_quads[dev] : p.num_sms / 4;
-    }
+    if (cudaGetDevice(&dev) != cudaSuccess) return "no CUDA device";
+    Clusters n;
+    const char *refused = devices.get(dev, &n, [](Clusters *d) -> const char * {
+        const auto limit = [](const void *f, size_t bytes) {
+            return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
+        };
+        if (setup_gemm<PEpiQKV>() != cudaSuccess || setup_gemm<PEpiResidual>() != cudaSuccess ||
+            setup_gemm<PEpiSwiGLU>() != cudaSuccess ||
+            !limit((const void *)attn_tc_kernel<128>, AttnSmem<128>::TOTAL + 1024) ||
+            !limit((const void *)attn_tc_kernel<64>, AttnSmem<64>::TOTAL + 1024))
+            return "cannot raise the shared-memory limits of the prefill kernels";
+        if (resident_clusters<PEpiSwiGLU>(2, &d->pairs) != cudaSuccess ||
+            resident_clusters<PEpiSwiGLU>(4, &d->quads) != cudaSuccess)
+            return "cannot query the resident clusters of the tensor-core GEMM";
+        return nullptr;
+    });
+    if (refused) return refused;
+    m->pairs = n.pairs < p.num_sms / 2 ? n.pairs : p.num_sms / 2;
+    m->quads = n.quads < p.num_sms / 4 ? n.quads : p.num_sms / 4;
     return nullptr;
 }
 

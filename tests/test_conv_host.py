@@ -1,5 +1,5 @@
-"""The convolution layer's host-side bookkeeping (csrc/conv_plan.h), compiled by itself with
-the host compiler: no GPU and no CUDA."""
+"""The convolution layer's host-side bookkeeping (csrc/conv_plan.h, csrc/device_table.h), compiled
+by itself with the host compiler: no GPU and no CUDA."""
 import os
 import shutil
 import subprocess
@@ -15,7 +15,7 @@ def run_host(tmp_path, body):
     if not cxx:
         pytest.skip("needs g++")
     src, exe = tmp_path / "t.cc", tmp_path / "t"
-    src.write_text('#include "conv_plan.h"\n#include <cstdio>\n#include <thread>\n#include <vector>\nusing namespace wici;\n'
+    src.write_text('#include "conv_plan.h"\n#include "device_table.h"\n#include <cstdio>\n#include <thread>\n#include <vector>\nusing namespace wici;\n'
                    '#define CHECK(x) do { if (!(x)) { std::printf("failed: %s\\n", #x); return 1; } } while (0)\n'
                    "int main() {\n" + body + "\nreturn 0;\n}\n")
     subprocess.run([cxx, "-std=c++17", "-O1", "-pthread", "-I", CSRC, str(src), "-o", str(exe)], check=True)
@@ -27,7 +27,7 @@ def test_each_device_keeps_its_own_counts(tmp_path):
     # two threads on two devices with different counts: each call gets its own device's, and a
     # device is asked once; a failed query is returned and asked again
     run_host(tmp_path, r"""
-    ConvDevices devs;
+    DeviceTable<ConvDevice> devs;
     int asked[2] = {0, 0};
     auto query = [&](int dev) {
         return [&asked, dev](ConvDevice *d) {
@@ -54,6 +54,10 @@ def test_each_device_keeps_its_own_counts(tmp_path):
     for (auto &t : threads) t.join();
     CHECK(wrong[0] == 0 && wrong[1] == 0);
     CHECK(asked[0] == 1 && asked[1] == 1);
+    // counts of zero are an answer like any other
+    int n = 0;
+    for (int i = 0; i < 2; ++i) CHECK(devs.get(2, &none, [&](ConvDevice *) { ++n; return 0; }) == 0 && none.sms == 0);
+    CHECK(n == 1);
     """)
 
 
