@@ -186,7 +186,6 @@ struct MEpiResidual {  // out[u] = prev[u] + v   (O projection, down projection)
     uint64_t *out;
     uint32_t tag;
     uint64_t pre;
-    static constexpr bool kArgmax = false;
     __device__ uint64_t base(int u) const {
         return embed ? tagged(bf16_to_f32(embed[u]), prev_tag) : ld_tagged(prev + u);
     }
@@ -203,7 +202,6 @@ struct MEpiResidual {  // out[u] = prev[u] + v   (O projection, down projection)
 struct MEpiSwiGLU {    // rows (2u, 2u+1) are (gate_u, up_u): m[u] = silu(g) * u
     uint64_t *m;
     uint32_t tag;
-    static constexpr bool kArgmax = false;
     __device__ void prefetch(int) {}
     __device__ void unit(int u, const float *v, bool) {
         const float gt = v[0];
@@ -211,7 +209,7 @@ struct MEpiSwiGLU {    // rows (2u, 2u+1) are (gate_u, up_u): m[u] = silu(g) * u
     }
 };
 
-// Packed QKV rows (pairs as in EpiQKV): q and k after RoPE (before their norms
+// Packed QKV rows (rows i and i + D/2 of a head are neighbours): q and k after RoPE (before their norms
 // with qk_norm) and v, in natural order; the attention phase stores K and V.
 template <int D>
 struct MEpiQKV {
@@ -222,7 +220,6 @@ struct MEpiQKV {
     int qkdim;
     bool raw;
     uint32_t pre;
-    static constexpr bool kArgmax = false;
     __device__ void prefetch(int u) {
         if (bias) pre = *reinterpret_cast<const uint32_t *>(bias + 2 * u);
     }
@@ -468,8 +465,8 @@ __device__ bool mc_gemv(MegaRing &R, float *red, int K, int n_units, int rpu, co
         if constexpr (!FULL) {
             // this thread's chunks of all RPS rows into registers (past the last row: old bytes of
             // the ring; no row's sum meets another's, and those are dropped), then the slot is free:
-            // its next copy need not wait for the products (steps of hidden 3072 414 -> 375 us,
-            // Qwen2.5-14B widths 637 -> 609, the 8-bit format at Qwen3-8B widths 524 -> 468)
+            // its next copy need not wait for the products (steps of hidden 3072 414 -> 367 us,
+            // Qwen2.5-14B widths 637 -> 597, the 8-bit format at Qwen3-8B widths 524 -> 470)
             uint4 w[RPS][NCH];
 #pragma unroll
             for (int r = 0; r < RPS; ++r)
@@ -485,7 +482,9 @@ __device__ bool mc_gemv(MegaRing &R, float *red, int K, int n_units, int rpu, co
 #pragma unroll
                 for (int j = 0; j < NCH; ++j) acc[r] = dot8(w[r][j], h[j], acc[r]);
             }
-        } else {   // without tails, loads and products interleaved are better (1B widths 520 us against 540)
+        } else {
+            // without tails, loads and products interleaved: measured better at the 1B widths (520 us
+            // against 540) and equal at the 8B ones, the two of these shapes that were tried
 #pragma unroll
             for (int r = 0; r < RPS; ++r) acc[r] = 0.f;
             if (!ok) {
@@ -746,8 +745,9 @@ __device__ __forceinline__ bool mc_phase(MegaRing &R, float *red, int K, int n_u
 // precision) and K and V are exact bf16, so every product is exact.  The sums are fp32
 // in the accumulators, O's over every page that a warp takes: its error against 64 bits
 // grows with them (8B widths, 8000 keys: 3.2e-7 at four pages a warp, 7.0e-7 at 63)
-// and stays below that of fp32 FMAs in its place (8.5e-7).  A scalar version (one warp per head and page, lane-transposed dot
-// products) took about 1 us per page: 29 us a layer at 8K cached tokens.
+// and stays below that of fp32 FMAs in its place (8.5e-7).  A scalar version (one warp per
+// head and page, lane-transposed dot products) took about 1 us per page: 29 us a layer at
+// 8K cached tokens.
 // The warps' states (O, m, l) are merged in shared memory and published as tagged
 // words; each CTA of the head then combines every split's states for its share
 // of the group's outputs.
@@ -1143,8 +1143,9 @@ __device__ inline void mega_rebalance(const MegaArgs &a, float *scr) {
 // partition.  Where a thread holds two or more chunks of every hidden-wide row (bf16 rows of
 // more than 2048 elements in a named shape), the step is launched with twelve warps of 168
 // and the producer's warpgroup hands its own on: 384 x 168 = 128 x 104 + 256 x 200.  The
-// compiler then keeps more loads of a phase in flight: Llama-3-8B widths, 2 layers and
-// 6360 tokens of context, 180 us a step -> 176; 14B widths, 6 layers, 599 -> 580.  The other
+// compiler then keeps more loads of a phase in flight.  The line lies between the measured
+// shapes: Llama-3-8B widths, 2 layers and 6360 tokens of context, 180 us a step -> 176; 14B
+// widths, 6 layers, 599 -> 580 (hidden 4096 and 5120 are all that takes it).  The other
 // shapes lose with it (1B 518 -> 536 us, 8-bit Qwen3-8B 9 layers 471 -> 482, widths picked
 // at run time 366 -> 370) and keep nine warps.  A producer of 24 and consumers of 240
 // measured the same (174 to 176, 579).

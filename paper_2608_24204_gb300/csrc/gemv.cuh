@@ -25,10 +25,10 @@ namespace wici {
 enum : int { SITE_GEMV_EMPTY = 11, SITE_GEMV_FULL = 12, SITE_GEMV_DRAIN = 13 };
 
 struct GemvIn {
-    const uint16_t *W;      // rows of this matrix, [n_units * rpu][K]
-    int K, n_units, rpu, ups;
+    const uint16_t *W;      // rows of this matrix, [n_units][K]
+    int K, n_units;
     int stages;             // ring slots (<= kGemvMaxStages)
-    uint32_t slot_bytes;    // bytes per ring slot (>= ups * rpu * K * 2, multiple of 128)
+    uint32_t slot_bytes;    // bytes per ring slot (>= gemv_rps(K) * K * 2, multiple of 128)
     const float *in;        // input vector (x when gain != nullptr)
     const uint16_t *gain;   // RMSNorm gain (bf16) or nullptr for a plain input
     int *ctrl;
@@ -48,7 +48,6 @@ struct EpiArgmax {    // logits[u] = v; greedy argmax (lowest index on ties) acr
     int pos_add;
     float best;
     int bidx;
-    static constexpr bool kArgmax = true;
     __device__ void unit(int u, const float *v) {
         logits[u] = v[0];
         if (v[0] > best || (v[0] == best && u < bidx)) {
@@ -72,16 +71,10 @@ static inline size_t gemv_smem_bytes(int stages, uint32_t slot_bytes) {
     return kGemvRedBytes + (size_t)stages * slot_bytes;
 }
 
-// ------------------------------------------------------------------- GEMV ----
-// Grid: num_sms CTAs, each owning a contiguous, balanced range of units.  Each
-// consumer thread holds NCH 8-element chunks of the input vector in registers
-// (chunk c = tid + 256 j) and, for every row of a stage, contributes the dot
-// product over its chunks; warp sums go to shared memory and are reduced over
-// the 8 warps (fixed order) once per batch of up to kRedRows rows.
-// Shapes: every slot holds RPS rows (RPS a power of two, at most 8, RPS x K x 2
-// <= 32 KB, a multiple of the unit); consumer thread t covers the 8-element
-// chunks c = t + 256 j, j < NCH; FULL when the chunks cover K exactly (no tail
-// check in the inner loop).
+// ------------------------------------------------------------ GEMV shapes ----
+// (NCH, RPS, FULL): every slot holds RPS rows (a power of two, at most 8, RPS x K x 2 <=
+// 32 KB); consumer thread t covers the 8-element chunks c = t + 256 j, j < NCH; FULL when
+// the chunks cover K exactly (no tail check in the inner loop).
 __host__ __device__ constexpr int gemv_rps(int K) {
     return 2 * K * 8 <= 32768 ? 8 : 2 * K * 4 <= 32768 ? 4 : 2 * K * 2 <= 32768 ? 2 : 1;
 }
@@ -249,12 +242,11 @@ __device__ inline bool lm_argmax(const EpiArgmax &e, float *s_bv, int *s_bi, int
 }
 
 // ------------------------------------------------------------------- GEMV ----
-// Grid: num_sms CTAs, each owning a contiguous, balanced range of units.  The
-// producer warp streams the CTA's rows, RPS per slot, through the ring; each of
-// the 8 consumer warps adds its chunks of every row and reduces the slot's RPS
-// rows with interleaved butterflies; warp sums go to shared memory and are
-// reduced over the warps (fixed order) once per kRedRows rows, then passed to
-// the epilogue.
+// Grid: num_sms CTAs, each owning a contiguous, balanced range of rows.  The producer warp
+// streams them, RPS per slot, through the ring; each consumer thread adds its chunks of
+// every row of a slot, each warp sums the slot's RPS rows with interleaved butterflies, and
+// the warp sums go to shared memory, where they are reduced over the 8 warps (fixed order)
+// once per batch of up to kRedRows rows and passed to the epilogue.
 template <int NCH, int RPS, bool FULL, class Epi>
 __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(const GemvIn g, const Epi epi_in) {
     extern __shared__ __align__(128) uint8_t smem[];
@@ -272,8 +264,7 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(const GemvIn g, c
     const int G = gridDim.x;
     const int u0 = (int)(((long long)blockIdx.x * g.n_units) / G);
     const int u1 = (int)(((long long)(blockIdx.x + 1) * g.n_units) / G);
-    const int nunits = u1 - u0;
-    const int total_rows = nunits * g.rpu;
+    const int total_rows = u1 - u0;
     const int nst = (total_rows + RPS - 1) / RPS;
     int *err = g.ctrl + CTRL_ERR;
 
@@ -293,7 +284,7 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(const GemvIn g, c
         if (lane == 0) {
             const uint64_t pol = l2_evict_first();
             const uint32_t ring0 = smem_u32(ring);
-            const uint16_t *src = g.W + (size_t)u0 * g.rpu * g.K;
+            const uint16_t *src = g.W + (size_t)u0 * g.K;
             int issued = 0;
             for (int s = 0; s < nst; ++s) {
                 const int slot = s % S;
@@ -418,25 +409,19 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(const GemvIn g, c
         if (s == nst - 1 || brow + RPS > kRedRows) {
             consumer_sync();
             if (s_abort) break;
-            const int bunits = brow / g.rpu;
-            for (int t = tid; t < bunits; t += kGemvConsumers) {
-                float v[2];
-                for (int j = 0; j < g.rpu; ++j) {
-                    float sum = 0.f;
+            for (int t = tid; t < brow; t += kGemvConsumers) {
+                float v = 0.f;
 #pragma unroll
-                    for (int w = 0; w < kGemvWarps; ++w)
-                        sum += red[(size_t)(buf * kGemvWarps + w) * kRedRows + t * g.rpu + j];
-                    v[j] = sum;
-                }
-                epi.unit(u0 + bunit0 + t, v);
+                for (int w = 0; w < kGemvWarps; ++w) v += red[(size_t)(buf * kGemvWarps + w) * kRedRows + t];
+                epi.unit(u0 + bunit0 + t, &v);
             }
-            bunit0 += bunits;
+            bunit0 += brow;
             brow = 0;
             buf ^= 1;
         }
     }
 
-    if constexpr (Epi::kArgmax) lm_argmax(epi, s_bv, s_bi, &s_last);
+    lm_argmax(epi, s_bv, s_bi, &s_last);
 }
 
 }  // namespace wici

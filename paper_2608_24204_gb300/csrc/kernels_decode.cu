@@ -90,7 +90,6 @@ cudaError_t setup_kernels() {
 // Ring geometry: slots of gemv_rps(K) rows, as many as fit kGemvRingBytes (2 to 8).
 static void ring_geometry(GemvIn &g) {
     const int rps = gemv_rps(g.K);
-    g.ups = rps / g.rpu;
     g.slot_bytes = ((uint32_t)rps * (uint32_t)g.K * 2u + 127u) & ~127u;
     int st = (int)(kGemvRingBytes / g.slot_bytes);
     g.stages = st < 2 ? 2 : (st > kGemvMaxStages ? kGemvMaxStages : st);
@@ -100,7 +99,7 @@ static cudaError_t launch_lm_head(GemvIn g, float *logits, int2 *partials, int *
                                   cudaStream_t st, bool pdl) {
     ring_geometry(g);
     void *fn = gemv_fn<EpiArgmax>(g.K);
-    if (!fn || g.ups < 1) return cudaErrorInvalidValue;
+    if (!fn) return cudaErrorInvalidValue;
     EpiArgmax e = {};
     e.logits = logits;
     e.partial = partials;
@@ -118,7 +117,6 @@ static GemvIn lm_head_in(const uint16_t *W, const uint16_t *gain, const float *x
     g.W = W;
     g.K = H;
     g.n_units = V;
-    g.rpu = 1;
     g.in = x;
     g.gain = gain;
     g.ctrl = ctrl;

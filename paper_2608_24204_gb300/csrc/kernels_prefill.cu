@@ -2,7 +2,7 @@
 // layer.  The four linear maps of a layer run on the tcgen05 GEMM (gemm_tc.cuh)
 // with fused epilogues (bias + RoPE + paged KV append, residual add, SwiGLU)
 // and the causal attention on the tcgen05 attention kernel (attn_tc.cuh); the
-// kernels around them produce the tensor-core operands as bf16 hi/lo pairs.
+// kernels around them produce the tensor-core operands as bf16 terms (split_bf16x3).
 #include <cuda.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -224,15 +224,9 @@ bool encode_tiled(CUtensorMap *m, int rank, const void *ptr, const uint64_t *dim
 
 // 2-D map over a row-major bf16 matrix [rows][K]; boxes of 64 x box_rows, 128 B swizzle
 static bool encode_2d(CUtensorMap *m, const void *ptr, int rows, int K, int box_rows) {
-    EncodeTiledFn enc = encode_fn();
-    if (!enc) return false;
-    cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)K * 2};
-    cuuint32_t box[2] = {(cuuint32_t)TC_BK, (cuuint32_t)box_rows};
-    cuuint32_t es[2] = {1, 1};
-    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(ptr), dims, strides, box, es,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    const uint64_t dims[2] = {(uint64_t)K, (uint64_t)rows}, strides[1] = {(uint64_t)K * 2};
+    const uint32_t box[2] = {(uint32_t)TC_BK, (uint32_t)box_rows}, es[2] = {1, 1};
+    return encode_tiled(m, 2, ptr, dims, strides, box, es);
 }
 
 const CUtensorMap *matrix_map(const MatrixMaps &m, int box) {
@@ -255,17 +249,11 @@ static MatrixMaps matrix(const void *ptr, int rows, int K) {
 // the KV pool of every layer as [page (layer-major)][K|V][kv head][16 slots][d]:
 // boxes of 64 d x 16 slots of one (page, K|V, head)
 static bool encode_kv(CUtensorMap *m, const void *ptr, const Plan &p) {
-    EncodeTiledFn enc = encode_fn();
-    if (!enc) return false;
-    cuuint64_t dims[5] = {(cuuint64_t)p.d, (cuuint64_t)kPage, (cuuint64_t)p.nkv, 2,
-                          (cuuint64_t)p.L * (cuuint64_t)p.max_pages};
-    cuuint64_t strides[4] = {(cuuint64_t)p.d * 2, (cuuint64_t)kPage * p.d * 2, (cuuint64_t)p.nkv * kPage * p.d * 2,
-                             (cuuint64_t)2 * p.nkv * kPage * p.d * 2};
-    cuuint32_t box[5] = {64, (cuuint32_t)kPage, 1, 1, 1};
-    cuuint32_t es[5] = {1, 1, 1, 1, 1};
-    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void *>(ptr), dims, strides, box, es,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    const uint64_t dims[5] = {(uint64_t)p.d, (uint64_t)kPage, (uint64_t)p.nkv, 2, (uint64_t)p.L * (uint64_t)p.max_pages};
+    const uint64_t strides[4] = {(uint64_t)p.d * 2, (uint64_t)kPage * p.d * 2, (uint64_t)p.nkv * kPage * p.d * 2,
+                                 (uint64_t)2 * p.nkv * kPage * p.d * 2};
+    const uint32_t box[5] = {64, (uint32_t)kPage, 1, 1, 1}, es[5] = {1, 1, 1, 1, 1};
+    return encode_tiled(m, 5, ptr, dims, strides, box, es);
 }
 
 const char *make_prefill_maps(const Plan &p, const Bufs &b, PrefillMaps *m) {

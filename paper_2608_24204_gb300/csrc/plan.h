@@ -21,7 +21,6 @@ constexpr int kGemvThreads = 288;  // 8 consumer warps + 1 producer warp
 #endif
 constexpr uint32_t kGemvRingBytes = WICI_GEMV_RING_BYTES;   // shared-memory ring per CTA
 constexpr int kGemvCtasPerSm = WICI_GEMV_CTAS_PER_SM;       // GEMV grid = SMs x this
-constexpr uint32_t kGemvStageMax = 32768;  // one unit (<= 2 rows of hidden <= 8192, or a row of K <= 16384)
 
 // Bytes of one matrix row of K input columns in the 8-bit block format as the
 // decode kernel streams it: K int8 codes followed by the row's K/32 fp16 block

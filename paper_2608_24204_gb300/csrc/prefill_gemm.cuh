@@ -85,7 +85,6 @@ struct Terms {   // kTerms pointers passed by value to kernels
 // --------------------------------------------------------------- epilogues ----
 // pair(t, c, a, b): GEMM output row t, columns (c, c + 1)
 struct PEpiQKV {  // packed QKV columns -> Q (three bf16 terms) and K/V pages (bf16)
-    static constexpr bool kRow = true;
     static constexpr int kATerms = kTerms;   // activation terms the GEMM multiplies
     Terms Q;
     uint16_t *kv;
@@ -217,7 +216,6 @@ struct PEpiQKV {  // packed QKV columns -> Q (three bf16 terms) and K/V pages (b
 struct PEpiResidual {  // X[t][c] += v
     float *X;
     int ld;
-    static constexpr bool kRow = true;
     // the O and down GEMMs multiply two terms of their activations (o, m): with
     // gate/up also at two terms, measured at 1.36e-2 max-abs against the fp64
     // oracle at the Qwen2.5-14B shape (1.30e-2 with three); the QKV GEMM keeps
@@ -252,7 +250,6 @@ struct PEpiResidual {  // X[t][c] += v
 struct PEpiSwiGLU {  // interleaved (gate, up) columns -> M[t][c/2] = silu(g) * u as three terms
     Terms M;
     int ld;
-    static constexpr bool kRow = true;
     // the gate/up GEMM multiplies two terms of its activation (16 significant bits):
     // measured against the fp64 oracle at the 8B and 14B shapes, it moves the
     // logits by less than 1e-4, where two terms in every GEMM fail the tolerance

@@ -312,13 +312,14 @@ int wici_create(const wici_config *cfg, void *cuda_stream, void *weight_dev, voi
     if (c->plan.qk_norm && !decode_has_named_shape(c->plan)) {
         delete c;
         return fail(nullptr, WICI_E_ARG,
-                    "config: the per-head q/k norm is built into the one-launch decode step, which needs "
-                    "n_q_heads * head_dim == hidden and an instantiated width");
+                    "config: the per-head q/k norm is built for n_q_heads * head_dim == hidden and, with head_dim 128, "
+                    "hidden 4096 / ffn 14336 or 12288 and hidden 5120 / ffn 13824, with head_dim 64, hidden 2048 / "
+                    "ffn 8192 and hidden, ffn below 2048");
     }
     if (c->plan.q8 && !decode_has_named_shape(c->plan)) {
         delete c;
         return fail(nullptr, WICI_E_ARG,
-                    "config: the 8-bit block format is built for hidden 4096 / ffn 14336 (head_dim 128) and for "
+                    "config: the 8-bit block format is built for hidden 4096 / ffn 14336 or 12288 (head_dim 128) and for "
                     "hidden, ffn below 2048 (head_dim 64), with n_q_heads * head_dim == hidden");
     }
     c->device = dev;
