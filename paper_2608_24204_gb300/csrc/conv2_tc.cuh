@@ -6,9 +6,9 @@
 // 32 KB instead of 48, so the ring holds six.  Same products in the same order as
 // conv_tc.cuh.  Barriers and roles as in gemm2_tc.cuh.
 //
-// Measured at the paper's sample (4 x 1024 x 224 x 224, 1024 filters; 947 GFLOP each), us,
-// one CTA per tile (with 16-byte stores) and pairs (with 32-byte ones): forward 581 and
-// 539, data gradient 836 and 633, filter gradient 709 and 685.
+// Measured at the paper's sample (4 x 1024 x 224 x 224, 1024 filters; 947 GFLOP each), us a
+// call, one CTA per tile (with 16-byte stores) and pairs (with 32-byte ones): forward 587 and
+// 540, data gradient (with the filter's transposition) 845 and 637, filter gradient 716 and 655.
 #pragma once
 #include "conv_tc.cuh"
 #include "gemm2_tc.cuh"

@@ -1,7 +1,9 @@
 // The decode step for widths without an instantiation of their own (bf16): the same
 // persistent kernel with each phase's shape picked at run time.  Such widths used to run
 // as five launches a layer and the LM head, 77 us a layer at hidden 3072, ffn 8192 (24
-// heads of 128), against 41 here and 30 of HBM time.
+// heads of 128), against 41 here and 30 of HBM time.  Eight bodies for each of five phases in one kernel spill
+// (1.1 to 1.2 KB a thread); twelve warps with 200 registers each take the spills away and
+// are no faster (367 to 373 us a step against 366), so the step keeps nine warps.
 #include "decode_step.cuh"
 
 namespace wici {
